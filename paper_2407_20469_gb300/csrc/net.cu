@@ -9,9 +9,9 @@
 //   | dense 258->256, ReLU | dense 256->12 (Noll 4..15).
 // Weights and the activations that feed a layer are BF16, products accumulate
 // in FP32 on the tensor cores (mma.sync m16n8k16), gradients and the AdamW
-// master weights are FP32. Every convolution (forward, data gradient, weight
-// gradient) and dense layer is one generic GEMM kernel whose operands are
-// gathered through loader functors (implicit im2col), with split-K and atomic
+// master weights are FP32. The convolutions (forward with ReLU, pool or mean; data and
+// weight gradients) are the kernels of netconv.cuh; the dense layers one generic GEMM
+// kernel whose operands are gathered through loader functors, with split-K and atomic
 // accumulation for the weight gradients.
 //
 // Parameters: six matrices W_l [out_l][taps_l + 1] stored back to back in FP32,
@@ -28,7 +28,9 @@
 
 #include "../../include/apic.h"
 #include "internal.cuh"
+#include "netconv.cuh"
 #include "regfft.cuh"
+#include "rowsum.cuh"
 
 namespace apic {
 namespace net {
@@ -96,13 +98,20 @@ __global__ void __launch_bounds__(512, 1) k_features(DevPlan P, int n_tiles, con
     for (int prob = blockIdx.x; prob < nprob; prob += gridDim.x) {
         const int tile = prob / kIn, i = prob - tile * kIn;
         const float* img = I + ((size_t)tile * P.n_img + i) * n * n;
-        double s = 0;
+        // the image's sum: per thread as a float pair (rowsum.cuh; an FP64 add per pixel kept
+        // the FP64 pipe busy for a quarter of the kernel's time), across threads in FP64
+        FF sum = {0.f, 0.f};
         const float4* img4 = reinterpret_cast<const float4*>(img);
         for (int q = threadIdx.x; q < n * n / 4; q += blockDim.x) {
             const float4 v = img4[q];
-            s += (double)v.x + v.y + v.z + v.w;
+            const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const FF t = ff_two_sum(sum.hi, x[e]);
+                sum = {t.hi, sum.lo + t.lo};
+            }
         }
-        s = block_sum(s, red);
+        const double s = block_sum((double)sum.hi + (double)sum.lo, red);
         const float inv_dc = s > 0 ? (float)(1.0 / s) : 0.f;
         for (int r = hw; r < n; r += NHW) {
             float2 v[BN], o[S][16];
@@ -154,14 +163,6 @@ size_t features_smem(int BN) {
 // epilogue must then accumulate atomically).
 constexpr int kBM = 64, kBN = 64, kBK = 32, kLD = kBK + 8;
 
-__device__ __forceinline__ void mma_bf16(float (&d)[4], const unsigned (&a)[4], const unsigned (&b)[2]) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};\n"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
 // Staging of 16 consecutive k of one A row (m fixed) or one B column (n fixed)
 // into 16 BF16 values of shared memory (16-byte aligned). Loaders whose data is
 // contiguous along k provide segA / segB with vector loads; the others go
@@ -180,17 +181,6 @@ struct HasSegB<F, std::void_t<decltype(std::declval<const F&>().segB(0, 0, 0, (_
 __device__ __forceinline__ void zero16(__nv_bfloat16* dst) {
     reinterpret_cast<uint4*>(dst)[0] = make_uint4(0, 0, 0, 0);
     reinterpret_cast<uint4*>(dst)[1] = make_uint4(0, 0, 0, 0);
-}
-
-__device__ __forceinline__ unsigned pack_bf16(float a, float b) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<const unsigned*>(&h);
-}
-
-// 8 floats (two float4, 16-byte aligned source) -> 8 BF16 (one uint4)
-__device__ __forceinline__ uint4 f8_to_bf16(const float* src) {
-    const float4 a = reinterpret_cast<const float4*>(src)[0], b = reinterpret_cast<const float4*>(src)[1];
-    return make_uint4(pack_bf16(a.x, a.y), pack_bf16(a.z, a.w), pack_bf16(b.x, b.y), pack_bf16(b.z, b.w));
 }
 
 template <class F>
@@ -260,7 +250,7 @@ __global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, int k_split, 
 #pragma unroll
             for (int i = 0; i < 2; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], a[i], b[j]);
+                for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], a[i], b[j][0], b[j][1]);
         }
         __syncthreads();
     }
@@ -294,124 +284,6 @@ cudaError_t gemm(int M, int N, int K, int splits, LA la, LB lb, EP ep, cudaStrea
 __device__ __forceinline__ float to_f(float v) { return v; }
 __device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
 
-// im2col of an NHWC H x H map with C channels for a 3x3, pad-1 convolution:
-// (m, k) with m = (b, y, x) and k = (dy, dx, c); k = 9 C is the bias column.
-// Serves as A of the forward pass and, called as (pixel, tap), as B of the
-// weight gradient.
-template <int H, int C, class T>
-struct ConvIn {
-    const T* x;
-    __device__ float operator()(int m, int k) const {
-        if (k >= 9 * C) return 1.f;
-        const int c = k % C, s = k / C, dy = s / 3, dx = s - 3 * dy;
-        const int q = m / H, xx = m - q * H + dx - 1;
-        const int b = q / H, yy = q - b * H + dy - 1;
-        if ((unsigned)yy >= (unsigned)H || (unsigned)xx >= (unsigned)H) return 0.f;
-        return to_f(x[(((size_t)b * H + yy) * H + xx) * C + c]);
-    }
-    // address of channel c of tap s at output pixel m, or NULL in the padding
-    __device__ const T* tap(int m, int s, int c) const {
-        const int dy = s / 3, dx = s - 3 * dy;
-        const int q = m / H, xx = m - q * H + dx - 1;
-        const int b = q / H, yy = q - b * H + dy - 1;
-        if ((unsigned)yy >= (unsigned)H || (unsigned)xx >= (unsigned)H) return nullptr;
-        return x + (((size_t)b * H + yy) * H + xx) * C + c;
-    }
-    // 16 consecutive taps of a row: one tap's 16 channels (C % 16 == 0, BF16
-    // maps) or two taps' 8 channels (C == 8, FP32 input); vector loads
-    __device__ void segA(int m, int k0, int kend, __nv_bfloat16* dst) const {
-        if (k0 + 16 <= kend && k0 + 16 <= 9 * C) {
-            if constexpr (std::is_same<T, __nv_bfloat16>::value && C % 16 == 0) {
-                const int s = k0 / C;
-                const T* p = tap(m, s, k0 - s * C);
-                if (p) {
-                    reinterpret_cast<uint4*>(dst)[0] = reinterpret_cast<const uint4*>(p)[0];
-                    reinterpret_cast<uint4*>(dst)[1] = reinterpret_cast<const uint4*>(p)[1];
-                } else {
-                    zero16(dst);
-                }
-                return;
-            } else if constexpr (std::is_same<T, float>::value && C == 8) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const T* p = tap(m, k0 / 8 + h, 0);
-                    reinterpret_cast<uint4*>(dst)[h] = p ? f8_to_bf16(p) : make_uint4(0, 0, 0, 0);
-                }
-                return;
-            }
-        }
-#pragma unroll 4
-        for (int c = 0; c < 16; ++c) dst[c] = __float2bfloat16(k0 + c < kend ? (*this)(m, k0 + c) : 0.f);
-    }
-};
-// (co, pixel) of the pre-activation gradient dz = dr * [r > 0]
-template <int C>
-struct ReluGradT {
-    const float* g;
-    const __nv_bfloat16* r;
-    __device__ float operator()(int c, int m) const {
-        const size_t i = (size_t)m * C + c;
-        return __bfloat162float(r[i]) > 0.f ? g[i] : 0.f;
-    }
-};
-// data gradient of the convolution: (m, k) with m = (b, y, x) of the input map
-// and k = (dy, dx, co) reads dz at (y - dy + 1, x - dx + 1)
-template <int H, int Co>
-struct DzShift {
-    const float* g;
-    const __nv_bfloat16* r;
-    __device__ float operator()(int m, int k) const {
-        const int co = k % Co, s = k / Co, dy = s / 3, dx = s - 3 * dy;
-        const int q = m / H, xx = m - q * H - dx + 1;
-        const int b = q / H, yy = q - b * H - dy + 1;
-        if ((unsigned)yy >= (unsigned)H || (unsigned)xx >= (unsigned)H) return 0.f;
-        const size_t i = (((size_t)b * H + yy) * H + xx) * Co + co;
-        return __bfloat162float(r[i]) > 0.f ? g[i] : 0.f;
-    }
-    // 16 consecutive output channels of one tap (Co % 16 == 0): vector loads of
-    // the gradient and of the activation that masks it
-    __device__ void segA(int m, int k0, int kend, __nv_bfloat16* dst) const {
-        static_assert(Co % 16 == 0, "16 channels per segment");
-        if (k0 + 16 <= kend) {
-            const int s = k0 / Co, co = k0 - s * Co, dy = s / 3, dx = s - 3 * dy;
-            const int q = m / H, xx = m - q * H - dx + 1;
-            const int b = q / H, yy = q - b * H - dy + 1;
-            if ((unsigned)yy >= (unsigned)H || (unsigned)xx >= (unsigned)H) {
-                zero16(dst);
-                return;
-            }
-            const size_t i = (((size_t)b * H + yy) * H + xx) * Co + co;
-            const float4* g4 = reinterpret_cast<const float4*>(g + i);
-            const uint4* r4 = reinterpret_cast<const uint4*>(r + i);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const uint4 rv = r4[h];
-                const __nv_bfloat16* rb = reinterpret_cast<const __nv_bfloat16*>(&rv);
-                const float4 a = g4[2 * h], c = g4[2 * h + 1];
-                const float v[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
-                unsigned w[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    w[e] = pack_bf16(__bfloat162float(rb[2 * e]) > 0.f ? v[2 * e] : 0.f,
-                                     __bfloat162float(rb[2 * e + 1]) > 0.f ? v[2 * e + 1] : 0.f);
-                reinterpret_cast<uint4*>(dst)[h] = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-            return;
-        }
-#pragma unroll 4
-        for (int c = 0; c < 16; ++c) dst[c] = __float2bfloat16(k0 + c < kend ? (*this)(m, k0 + c) : 0.f);
-    }
-};
-// (k = (dy, dx, co), n = ci) -> W[co][(dy, dx, ci)]
-template <int Ci, int Co>
-struct WFlip {
-    const __nv_bfloat16* w;
-    int ld;
-    __device__ float operator()(int k, int n) const {
-        const int co = k % Co, s = k / Co;
-        return __bfloat162float(w[(size_t)co * ld + s * Ci + n]);
-    }
-};
 struct WT {                 // B(k, n) = W[n][k]; rows padded to multiples of 8
     const __nv_bfloat16* w;
     int ld;
@@ -459,14 +331,6 @@ struct MatBias {            // (r, c) -> p[r][c], 1 in column `cols` (bias colum
 };
 
 // ---- epilogues
-struct EpConv {             // r = relu(acc + bias) as bf16, [m][ld]
-    __nv_bfloat16* out;
-    const float* bias;
-    int bias_stride, ld;
-    __device__ void operator()(int m, int n, float v) const {
-        out[(size_t)m * ld + n] = __float2bfloat16(fmaxf(v + bias[(size_t)n * bias_stride], 0.f));
-    }
-};
 struct EpDense {            // fp32 acc + bias, optional ReLU
     float* out;
     const float* bias;
@@ -475,6 +339,30 @@ struct EpDense {            // fp32 acc + bias, optional ReLU
     __device__ void operator()(int m, int n, float v) const {
         const float r = v + bias[(size_t)n * bias_stride];
         out[(size_t)m * ld + n] = relu ? fmaxf(r, 0.f) : r;
+    }
+};
+struct EpOut {              // the network's outputs: fp32 acc + bias to y, and Noll 1..15 (1..3 zero) to out15
+    float* y;
+    float* out15;
+    const float* bias;
+    int bias_stride;
+    __device__ void operator()(int m, int n, float v) const {
+        const float r = v + bias[(size_t)n * bias_stride];
+        y[(size_t)m * kOut + n] = r;
+        if (out15) {
+            float* o = out15 + (size_t)m * APIC_N_ZERNIKE;
+            o[n + 3] = r;
+            if (n < 3) o[n] = 0.f;
+        }
+    }
+};
+struct EpMask {             // gradient of a ReLU's input: v where its output h is positive
+    float* out;
+    const float* h;
+    int ld;
+    __device__ void operator()(int m, int n, float v) const {
+        const size_t i = (size_t)m * ld + n;
+        out[i] = h[i] > 0.f ? v : 0.f;
     }
 };
 struct EpStore {
@@ -489,67 +377,6 @@ struct EpAtomic {
 };
 
 // ------------------------------------------------------------------ other layers
-// 2 x 2 max-pool of an NHWC bf16 map (first maximum in (dy, dx) order), with the
-// chosen position kept for the backward pass.
-__global__ void k_maxpool(const __nv_bfloat16* __restrict__ r, __nv_bfloat16* __restrict__ out,
-                          uint8_t* __restrict__ arg, int B, int H, int C) {
-    const int Ho = H / 2;
-    const size_t total = (size_t)B * Ho * Ho * C;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % C);
-        const size_t q = i / C;
-        const int x = (int)(q % Ho), y = (int)((q / Ho) % Ho), b = (int)(q / ((size_t)Ho * Ho));
-        float best = -INFINITY;
-        int bi = 0;
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            const float v = __bfloat162float(r[(((size_t)b * H + 2 * y + (s >> 1)) * H + 2 * x + (s & 1)) * C + c]);
-            if (v > best) {
-                best = v;
-                bi = s;
-            }
-        }
-        out[i] = __float2bfloat16(best);
-        arg[i] = (uint8_t)bi;
-    }
-}
-
-__global__ void k_maxpool_back(const float* __restrict__ g, const uint8_t* __restrict__ arg, float* __restrict__ gin,
-                               int B, int H, int C) {
-    const int Ho = H / 2;
-    const size_t total = (size_t)B * Ho * Ho * C;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % C);
-        const size_t q = i / C;
-        const int x = (int)(q % Ho), y = (int)((q / Ho) % Ho), b = (int)(q / ((size_t)Ho * Ho));
-        const int a = arg[i];
-#pragma unroll
-        for (int s = 0; s < 4; ++s)
-            gin[(((size_t)b * H + 2 * y + (s >> 1)) * H + 2 * x + (s & 1)) * C + c] = s == a ? g[i] : 0.f;
-    }
-}
-
-// global mean over the HW pixels of the last ReLU map, then (u, v)
-__global__ void k_gap_concat(const __nv_bfloat16* __restrict__ r, const float* __restrict__ uv,
-                             float* __restrict__ hin, int HW, int C) {
-    const int b = blockIdx.x;
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-        float s = 0.f;
-        for (int p = 0; p < HW; ++p) s += __bfloat162float(r[((size_t)b * HW + p) * C + c]);
-        hin[(size_t)b * (C + 2) + c] = s / (float)HW;
-    }
-    if (threadIdx.x < 2) hin[(size_t)b * (C + 2) + C + threadIdx.x] = uv ? uv[2 * b + threadIdx.x] : 0.f;
-}
-
-__global__ void k_gap_back(const float* __restrict__ ghin, float* __restrict__ gr, int B, int HW, int C) {
-    const size_t total = (size_t)B * HW * C;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % C);
-        const int b = (int)(i / ((size_t)HW * C));
-        gr[i] = ghin[(size_t)b * (C + 2) + c] / (float)HW;
-    }
-}
-
 // mean squared error over the batch and the 12 outputs (Noll 4..15 of the
 // [b][15] targets) and its gradient
 __global__ void k_loss(const float* __restrict__ y, const float* __restrict__ target, float* __restrict__ gy,
@@ -564,18 +391,6 @@ __global__ void k_loss(const float* __restrict__ y, const float* __restrict__ ta
     }
     acc = block_sum(acc, red);
     if (threadIdx.x == 0 && loss) *loss = (float)(acc / (B * kOut));
-}
-
-__global__ void k_pack_out(const float* __restrict__ y, float* __restrict__ out, int B) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < B * APIC_N_ZERNIKE; i += gridDim.x * blockDim.x) {
-        const int b = i / APIC_N_ZERNIKE, j = i - b * APIC_N_ZERNIKE;
-        out[i] = j < 3 ? 0.f : y[(size_t)b * kOut + j - 3];
-    }
-}
-
-__global__ void k_relu_mask(float* __restrict__ g, const float* __restrict__ h, size_t n) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        if (!(h[i] > 0.f)) g[i] = 0.f;
 }
 
 __global__ void k_cast_bf16(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, size_t n, Layout L) {
@@ -655,7 +470,7 @@ struct apic_net {
     uint8_t* arg[3] = {};
     float *hin = nullptr, *h4 = nullptr, *y = nullptr;
     // gradients of activations
-    float *g_r[4] = {}, *g_pool[3] = {}, *g_hin = nullptr, *g_h4 = nullptr, *g_y = nullptr;
+    float *g_pool[3] = {}, *g_hin = nullptr, *g_h4 = nullptr, *g_y = nullptr;
     long long launches = 0;
     std::vector<void*> allocs;
 };
@@ -684,8 +499,53 @@ bool nalloc(apic_net* n, T** p, size_t count) {
     return true;
 }
 
-// split-K factor of a weight-gradient GEMM: ~256 pixels per block, so even the small
-// late layers spread over a few thousand blocks
+// Launch shapes of the layers' kernels: blocks along the pixels of an image (or of the
+// images of one tile), and along the output and input channels
+template <class Cfg, int TILES, int GY, int GZ = 1>
+struct Layer {
+    using C = Cfg;
+    enum { tiles = TILES, gy = GY, gz = GZ };                    // tiles: blocks along the pixels, per image
+};
+// forward: 128 or 256 pixels x 32 or 64 channels per block (64 x 64 for the last layer's 8 x 8 maps)
+using C1 = Layer<ConvCfg<64, kC0, kC1, 32, 4, 8, 1>, 16, 1>;
+using C2 = Layer<ConvCfg<32, kC1, kC2, 64, 4, 4, 2>, 8, 1>;
+using C3 = Layer<ConvCfg<16, kC2, kC3, 64, 8, 4, 2>, 2, 2>;
+using C4 = Layer<ConvCfg<8, kC3, kC4, 64, 8, 2, 2>, 1, 4>;
+using D3 = Layer<DgradCfg<8, kC3, kC4, 32, 8>, 1, 4>;
+using D2 = Layer<DgradCfg<16, kC2, kC3, 64, 4>, 4, 1>;
+using D1 = Layer<DgradCfg<32, kC1, kC2, 32, 4>, 8, 1>;
+// weight gradients: tiles counted per IMG images
+using W3 = Layer<WgradCfg<8, kC3, kC4, 64, 64, 8, 2>, 1, 4, 2>;
+using W2 = Layer<WgradCfg<16, kC2, kC3, 64, 64, 8, 1>, 2, 2, 1>;
+using W1 = Layer<WgradCfg<32, kC1, kC2, 32, 64, 4, 1>, 8, 1, 1>;
+using W0 = Layer<WgradCfg<64, kC0, kC1, 8, 32, 4, 1>, 16, 1, 1>;
+
+template <class L, class K, class... A>
+cudaError_t launch_layer(K kernel, dim3 grid, int threads, long long* launches, cudaStream_t st, A... args) {
+    cudaError_t e = cudaSuccess;
+    if (L::C::smem > 48 * 1024) e = raise_smem_limit((const void*)kernel, L::C::smem);
+    if (e != cudaSuccess) return e;
+    kernel<<<grid, threads, L::C::smem, st>>>(args...);
+    ++*launches;
+    return cudaGetLastError();
+}
+template <class L, class K, class... A>
+cudaError_t conv(K kernel, int B, long long* launches, cudaStream_t st, A... args) {
+    return launch_layer<L>(kernel, dim3(B * L::tiles, L::gy), L::C::NTHR, launches, st, args...);
+}
+template <class L, class K, class... A>
+cudaError_t dgrad(K kernel, int B, long long* launches, cudaStream_t st, A... args) {
+    return launch_layer<L>(kernel, dim3(B * L::tiles, L::gy), 256, launches, st, args...);
+}
+// about two blocks per SM over all channel tiles: each adds its sums to the gradient once
+template <class L, class K, class... A>
+cudaError_t wgrad(K kernel, int B, long long* launches, cudaStream_t st, A... args) {
+    const int img = L::C::IMG, tiles = (B + img - 1) / img * L::tiles;
+    const int split = std::max(1, std::min<int>(tiles, L::C::target / (L::gy * L::gz)));
+    return launch_layer<L>(kernel, dim3(split, L::gy, L::gz), 256, launches, st, args...);
+}
+
+// split-K factor of a dense layer's weight-gradient GEMM
 int split_for(long long K) { return (int)std::max(1LL, std::min(512LL, K / 256)); }
 
 }  // namespace
@@ -701,38 +561,20 @@ cudaError_t net_predict(apic_net* n, int B, const float* feat, const float* uv, 
     cudaError_t e;
 #define NET_STEP(x)                          \
     if ((e = (x)) != cudaSuccess) return e;
-#define NET_POOL(l, H, C)                                                                                        \
-    k_maxpool<<<blocks_for((size_t)B * (H / 2) * (H / 2) * C), 256, 0, st>>>(n->r[l], n->pool[l], n->arg[l], B, H, \
-                                                                           C);                                    \
-    ++*nl;                                                                                                       \
-    NET_STEP(cudaGetLastError());
-    NET_STEP(gemm(B * 64 * 64, kC1, 9 * kC0, 1, ConvIn<64, kC0, float>{feat}, WT{n->wbf + L.offp[0], L.ldp(0)},
-                  EpConv{n->r[0], n->params + L.off[0] + L.taps[0], L.ld(0), kC1}, st, nl));
-    NET_POOL(0, 64, kC1);
-    NET_STEP(gemm(B * 32 * 32, kC2, 9 * kC1, 1, ConvIn<32, kC1, __nv_bfloat16>{n->pool[0]},
-                  WT{n->wbf + L.offp[1], L.ldp(1)}, EpConv{n->r[1], n->params + L.off[1] + L.taps[1], L.ld(1), kC2}, st,
+    auto wl = [&](int l) { return n->wbf + L.offp[l]; };
+    auto bl = [&](int l) { return n->params + L.off[l] + L.taps[l]; };
+    NET_STEP((conv<C1>(k_conv<64, kC0, kC1, 32, 4, 8, 1, true, float>, B, nl, st, feat, wl(0), L.ldp(0), bl(0), L.ld(0),
+                       n->r[0], n->pool[0], n->arg[0], nullptr, nullptr)));
+    NET_STEP((conv<C2>(k_conv<32, kC1, kC2, 64, 4, 4, 2, true, __nv_bfloat16>, B, nl, st, n->pool[0], wl(1), L.ldp(1),
+                       bl(1), L.ld(1), n->r[1], n->pool[1], n->arg[1], nullptr, nullptr)));
+    NET_STEP((conv<C3>(k_conv<16, kC2, kC3, 64, 8, 4, 2, true, __nv_bfloat16>, B, nl, st, n->pool[1], wl(2), L.ldp(2),
+                       bl(2), L.ld(2), n->r[2], n->pool[2], n->arg[2], nullptr, nullptr)));
+    NET_STEP((conv<C4>(k_conv<8, kC3, kC4, 64, 8, 2, 2, false, __nv_bfloat16>, B, nl, st, n->pool[2], wl(3), L.ldp(3),
+                       bl(3), L.ld(3), n->r[3], nullptr, nullptr, uv, n->hin)));
+    NET_STEP(gemm(B, kHidden, kHin, 1, Mat{n->hin, kHin}, WT{wl(4), L.ldp(4)},
+                  EpDense{n->h4, bl(4), L.ld(4), kHidden, true}, st, nl));
+    NET_STEP(gemm(B, kOut, kHidden, 1, Mat{n->h4, kHidden}, WT{wl(5), L.ldp(5)}, EpOut{n->y, out15, bl(5), L.ld(5)}, st,
                   nl));
-    NET_POOL(1, 32, kC2);
-    NET_STEP(gemm(B * 16 * 16, kC3, 9 * kC2, 1, ConvIn<16, kC2, __nv_bfloat16>{n->pool[1]},
-                  WT{n->wbf + L.offp[2], L.ldp(2)}, EpConv{n->r[2], n->params + L.off[2] + L.taps[2], L.ld(2), kC3}, st,
-                  nl));
-    NET_POOL(2, 16, kC3);
-    NET_STEP(gemm(B * 8 * 8, kC4, 9 * kC3, 1, ConvIn<8, kC3, __nv_bfloat16>{n->pool[2]},
-                  WT{n->wbf + L.offp[3], L.ldp(3)}, EpConv{n->r[3], n->params + L.off[3] + L.taps[3], L.ld(3), kC4}, st,
-                  nl));
-    k_gap_concat<<<B, 256, 0, st>>>(n->r[3], uv, n->hin, 64, kC4);
-    ++*nl;
-    NET_STEP(cudaGetLastError());
-    NET_STEP(gemm(B, kHidden, kHin, 1, Mat{n->hin, kHin}, WT{n->wbf + L.offp[4], L.ldp(4)},
-                  EpDense{n->h4, n->params + L.off[4] + L.taps[4], L.ld(4), kHidden, true}, st, nl));
-    NET_STEP(gemm(B, kOut, kHidden, 1, Mat{n->h4, kHidden}, WT{n->wbf + L.offp[5], L.ldp(5)},
-                  EpDense{n->y, n->params + L.off[5] + L.taps[5], L.ld(5), kOut, false}, st, nl));
-    if (out15) {
-        k_pack_out<<<(B * APIC_N_ZERNIKE + 255) / 256, 256, 0, st>>>(n->y, out15, B);
-        ++*nl;
-        NET_STEP(cudaGetLastError());
-    }
-#undef NET_POOL
 #undef NET_STEP
     return cudaSuccess;
 }
@@ -760,7 +602,7 @@ apic_status apic_net_create(int max_batch, apic_net** out) {
     const int C[4] = {kC1, kC2, kC3, kC4};
     int H = kCrop;
     for (int l = 0; l < 4 && ok; ++l) {
-        ok = nalloc(n, &n->r[l], B * H * H * C[l]) && nalloc(n, &n->g_r[l], B * H * H * C[l]);
+        ok = nalloc(n, &n->r[l], B * H * H * C[l]);
         if (ok && l < 3) {
             H /= 2;
             ok = nalloc(n, &n->pool[l], B * H * H * C[l]) && nalloc(n, &n->arg[l], B * H * H * C[l]) &&
@@ -884,49 +726,32 @@ apic_status apic_net_backward(apic_net* n, const float* target15, float* loss, v
     // dense 256 -> 12
     NET_TRY(gemm(kOut, L.ld(5), B, split_for(B), MatT{n->g_y, kOut}, MatBias{n->h4, kHidden, kHidden},
                  EpAtomic{n->grads + L.off[5], L.ld(5)}, st, nl));
-    NET_TRY(gemm(B, kHidden, kOut, 1, Mat{n->g_y, kOut}, WN{n->wbf + L.offp[5], L.ldp(5)}, EpStore{n->g_h4, kHidden},
-                 st, nl));
-    k_relu_mask<<<blocks_for((size_t)B * kHidden), 256, 0, st>>>(n->g_h4, n->h4, (size_t)B * kHidden);
-    ++*nl;
-    NET_TRY(cudaGetLastError());
+    NET_TRY(gemm(B, kHidden, kOut, 1, Mat{n->g_y, kOut}, WN{n->wbf + L.offp[5], L.ldp(5)},
+                 EpMask{n->g_h4, n->h4, kHidden}, st, nl));
     // dense 258 -> 256
     NET_TRY(gemm(kHidden, L.ld(4), B, split_for(B), MatT{n->g_h4, kHidden}, MatBias{n->hin, kHin, kHin},
                  EpAtomic{n->grads + L.off[4], L.ld(4)}, st, nl));
     NET_TRY(gemm(B, kHin, kHidden, 1, Mat{n->g_h4, kHidden}, WN{n->wbf + L.offp[4], L.ldp(4)}, EpStore{n->g_hin, kHin},
                  st, nl));
-    // global mean
-    k_gap_back<<<blocks_for((size_t)B * 64 * kC4), 256, 0, st>>>(n->g_hin, n->g_r[3], B, 64, kC4);
-    ++*nl;
-    NET_TRY(cudaGetLastError());
-    // conv 128 -> 256 on 8 x 8
-    NET_TRY(gemm(kC4, L.ld(3), B * 64, split_for(B * 64LL), ReluGradT<kC4>{n->g_r[3], n->r[3]},
-                 ConvIn<8, kC3, __nv_bfloat16>{n->pool[2]}, EpAtomic{n->grads + L.off[3], L.ld(3)}, st, nl));
-    NET_TRY(gemm(B * 64, kC3, 9 * kC4, 1, DzShift<8, kC4>{n->g_r[3], n->r[3]}, WFlip<kC3, kC4>{n->wbf + L.offp[3], L.ldp(3)},
-                 EpStore{n->g_pool[2], kC3}, st, nl));
-    k_maxpool_back<<<blocks_for((size_t)B * 64 * kC3), 256, 0, st>>>(n->g_pool[2], n->arg[2], n->g_r[2], B, 16, kC3);
-    ++*nl;
-    NET_TRY(cudaGetLastError());
-    // conv 64 -> 128 on 16 x 16
-    NET_TRY(gemm(kC3, L.ld(2), B * 256, split_for(B * 256LL), ReluGradT<kC3>{n->g_r[2], n->r[2]},
-                 ConvIn<16, kC2, __nv_bfloat16>{n->pool[1]}, EpAtomic{n->grads + L.off[2], L.ld(2)}, st, nl));
-    NET_TRY(gemm(B * 256, kC2, 9 * kC3, 1, DzShift<16, kC3>{n->g_r[2], n->r[2]}, WFlip<kC2, kC3>{n->wbf + L.offp[2], L.ldp(2)},
-                 EpStore{n->g_pool[1], kC2}, st, nl));
-    k_maxpool_back<<<blocks_for((size_t)B * 256 * kC2), 256, 0, st>>>(n->g_pool[1], n->arg[1], n->g_r[1], B, 32,
-                                                                     kC2);
-    ++*nl;
-    NET_TRY(cudaGetLastError());
-    // conv 32 -> 64 on 32 x 32
-    NET_TRY(gemm(kC2, L.ld(1), B * 1024, split_for(B * 1024LL), ReluGradT<kC2>{n->g_r[1], n->r[1]},
-                 ConvIn<32, kC1, __nv_bfloat16>{n->pool[0]}, EpAtomic{n->grads + L.off[1], L.ld(1)}, st, nl));
-    NET_TRY(gemm(B * 1024, kC1, 9 * kC2, 1, DzShift<32, kC2>{n->g_r[1], n->r[1]}, WFlip<kC1, kC2>{n->wbf + L.offp[1], L.ldp(1)},
-                 EpStore{n->g_pool[0], kC1}, st, nl));
-    k_maxpool_back<<<blocks_for((size_t)B * 1024 * kC1), 256, 0, st>>>(n->g_pool[0], n->arg[0], n->g_r[0], B, 64,
-                                                                      kC1);
-    ++*nl;
-    NET_TRY(cudaGetLastError());
-    // conv 8 -> 32 on 64 x 64 (weights only)
-    NET_TRY(gemm(kC1, L.ld(0), B * 4096, split_for(B * 4096LL), ReluGradT<kC1>{n->g_r[0], n->r[0]},
-                 ConvIn<64, kC0, float>{n->in}, EpAtomic{n->grads + L.off[0], L.ld(0)}, st, nl));
+    // convolutions, last first: weights, then the gradient of the layer's input
+    const DzMean<8, kC4> dz3{n->g_hin, kHin, n->r[3]};
+    const DzPool<16, kC3> dz2{n->g_pool[2], n->arg[2], n->pool[2]};
+    const DzPool<32, kC2> dz1{n->g_pool[1], n->arg[1], n->pool[1]};
+    const DzPool<64, kC1> dz0{n->g_pool[0], n->arg[0], n->pool[0]};
+    NET_TRY((wgrad<W3>(k_wgrad<8, kC3, kC4, 64, 64, 8, 2, 2, 4, 1, __nv_bfloat16, DzMean<8, kC4>>, B, nl, st, n->pool[2],
+                       dz3, B, n->grads + L.off[3])));
+    NET_TRY((dgrad<D3>(k_dgrad<8, kC3, kC4, 32, 8, 4, 2, DzMean<8, kC4>>, B, nl, st, dz3, n->wbf + L.offp[3], L.ldp(3),
+                       n->g_pool[2])));
+    NET_TRY((wgrad<W2>(k_wgrad<16, kC2, kC3, 64, 64, 8, 1, 2, 4, 1, __nv_bfloat16, DzPool<16, kC3>>, B, nl, st,
+                       n->pool[1], dz2, B, n->grads + L.off[2])));
+    NET_TRY((dgrad<D2>(k_dgrad<16, kC2, kC3, 64, 4, 4, 2, DzPool<16, kC3>>, B, nl, st, dz2, n->wbf + L.offp[2], L.ldp(2),
+                       n->g_pool[1])));
+    NET_TRY((wgrad<W1>(k_wgrad<32, kC1, kC2, 32, 64, 4, 1, 2, 4, 1, __nv_bfloat16, DzPool<32, kC2>>, B, nl, st,
+                       n->pool[0], dz1, B, n->grads + L.off[1])));
+    NET_TRY((dgrad<D1>(k_dgrad<32, kC1, kC2, 32, 4, 8, 1, DzPool<32, kC2>>, B, nl, st, dz1, n->wbf + L.offp[1], L.ldp(1),
+                       n->g_pool[0])));
+    NET_TRY((wgrad<W0>(k_wgrad<64, kC0, kC1, 8, 32, 4, 1, 1, 1, 8, float, DzPool<64, kC1>>, B, nl, st, n->in, dz0, B,
+                       n->grads + L.off[0])));
     return APIC_OK;
 }
 

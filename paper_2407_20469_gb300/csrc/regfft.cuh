@@ -20,6 +20,7 @@
 #include "common.cuh"
 
 namespace apic {
+inline namespace APIC_ARITH {
 
 // ---- compile-time cos / sin (Taylor series after reduction to [-pi/4, pi/4])
 namespace cx {
@@ -311,9 +312,11 @@ __device__ __forceinline__ void fft_beta2(float2 (&o)[16], float2 (&va)[B], floa
     __syncwarp(h.mask);
 }
 
+}  // inline namespace
 }  // namespace apic
 
 namespace apic {
+inline namespace APIC_ARITH {
 
 // ---- wide transforms: N = 16 B with 16 < B <= 32 (288, 320, 384, 512 points).
 // Step A is the same DFT_B in registers; step B has B DFT_16s, so lane t runs two
@@ -389,4 +392,5 @@ __device__ __forceinline__ void fft_b(float2 (&o)[Slots<B>::value][16], float2 (
         fft_beta<B, INV>(o[0], v, h, tw);
 }
 
+}  // inline namespace
 }  // namespace apic
