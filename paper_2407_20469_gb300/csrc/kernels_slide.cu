@@ -111,6 +111,7 @@ __global__ void k_blend_corr(int n_tiles, int cols, int u, int L, const float2* 
         const float2* ft = field + (size_t)k * L * L;
         const float2* fs = field + (size_t)nb * L * L;
         if (ya < yb && w > 0)
+#pragma unroll 4
             for (int idx = threadIdx.x; idx < (yb - ya) * w; idx += blockDim.x) {
                 const int Y = ya + idx / w, X = xa + idx % w;
                 const float2 a = ft[(size_t)(Y - ty) * L + (X - tx)], b = fs[(size_t)(Y - sy) * L + (X - sx)];
@@ -254,7 +255,7 @@ __global__ void k_blend(int rows, int cols, int u, int L, const float2* __restri
 // finds its column run and ramps once, and the block's first kBlendRows threads find the
 // row runs and ramps of the stripe into shared memory. A run longer than kMaxCover falls
 // back to the per-pixel rule.
-constexpr int kMaxCover = 4, kBlendThreads = 128, kBlendRows = 32;
+constexpr int kMaxCover = 4, kBlendThreads = 128, kBlendRows = 32, kBlendBatch = 4;
 
 // run of windows (starts u * start(0..count-1), increasing) covering p: last index and length
 // (length kMaxCover + 1 when longer than kMaxCover)
@@ -322,43 +323,70 @@ __global__ void __launch_bounds__(kBlendThreads) k_blend_pairs(int rows, int col
             wxb[c] = blend_ramp(sx, sp, sn, j > 0, j + 1 < cols, X + 1, L);
         }
     }
-#pragma unroll 2
-    for (int Y = Y0; Y < Y1; ++Y) {
-        const int r = Y - Y0, ni = s_n[r];
-        float4 o;
-        if (generic_x || ni < 0) {
-            const float2 a = blend_one(rows, cols, u, L, field, win, z, Y, X);
-            const float2 b = blend_one(rows, cols, u, L, field, win, z, Y, X + 1);
-            o = make_float4(a.x, a.y, b.x, b.y);
-        } else {
-            float ar0 = 0.f, ai0 = 0.f, ws0 = 0.f, ar1 = 0.f, ai1 = 0.f, ws1 = 0.f;
+    for (int Yb = Y0; Yb < Y1; Yb += kBlendBatch) {
+        // Pixels of one window only (its weight is 1) over the whole batch of rows, the
+        // bulk of a slide: the loads go out together and the phase is all there is to
+        // apply. The general rule costs some 120 instructions a row, four IEEE divisions
+        // among them. One call on a 16 x 32 window grid of 256: 641 -> 568 us. (Eight rows
+        // a batch with every row's first window loaded up front, whatever its weight, took
+        // 932 us: the general rule's registers halved the blocks in flight.)
+        bool single = nj == 1 && Yb + kBlendBatch <= Y1;
 #pragma unroll
-            for (int ci = 0; ci < kMaxCover; ++ci) {
-                if (ci < ni) {
-                    const int i = s_last[r] - ci, sy = s_sy[r][ci];
-                    const float wy = s_wy[r][ci];
+        for (int q = 0; q < kBlendBatch; ++q) single = single && s_n[Yb - Y0 + q] == 1;
+        if (single) {
+            float4 f[kBlendBatch];
+            float2 zk[kBlendBatch];
 #pragma unroll
-                    for (int c = 0; c < kMaxCover; ++c) {
-                        if (c < nj) {
-                            const int k = i * cols + jhi - c;
-                            const float4 f = __ldcs(reinterpret_cast<const float4*>(
-                                field + (size_t)k * L * L + (size_t)(Y - sy) * L + (X - sxs[c])));
-                            const float2 zk = z[k];
-                            const float w0 = wy * wxa[c], w1 = wy * wxb[c];
-                            ar0 += w0 * (f.x * zk.x - f.y * zk.y);
-                            ai0 += w0 * (f.x * zk.y + f.y * zk.x);
-                            ws0 += w0;
-                            ar1 += w1 * (f.z * zk.x - f.w * zk.y);
-                            ai1 += w1 * (f.z * zk.y + f.w * zk.x);
-                            ws1 += w1;
+            for (int q = 0; q < kBlendBatch; ++q) {
+                const int r = Yb - Y0 + q, k = s_last[r] * cols + jhi;
+                f[q] = __ldcs(reinterpret_cast<const float4*>(field + ((size_t)k * L + (Yb + q - s_sy[r][0])) * L +
+                                                              (X - sxs[0])));
+                zk[q] = z[k];
+            }
+#pragma unroll
+            for (int q = 0; q < kBlendBatch; ++q)
+                __stcs(reinterpret_cast<float4*>(out + (size_t)(Yb + q) * Wo + X),
+                       make_float4(f[q].x * zk[q].x - f[q].y * zk[q].y, f[q].x * zk[q].y + f[q].y * zk[q].x,
+                                   f[q].z * zk[q].x - f[q].w * zk[q].y, f[q].z * zk[q].y + f[q].w * zk[q].x));
+            continue;
+        }
+        for (int Y = Yb; Y < min(Yb + kBlendBatch, Y1); ++Y) {
+            const int r = Y - Y0, ni = s_n[r];
+            float4 o;
+            if (generic_x || ni < 0) {
+                const float2 a = blend_one(rows, cols, u, L, field, win, z, Y, X);
+                const float2 b = blend_one(rows, cols, u, L, field, win, z, Y, X + 1);
+                o = make_float4(a.x, a.y, b.x, b.y);
+            } else {
+                float ar0 = 0.f, ai0 = 0.f, ws0 = 0.f, ar1 = 0.f, ai1 = 0.f, ws1 = 0.f;
+#pragma unroll
+                for (int ci = 0; ci < kMaxCover; ++ci) {
+                    if (ci < ni) {
+                        const int i = s_last[r] - ci, sy = s_sy[r][ci];
+                        const float wy = s_wy[r][ci];
+#pragma unroll
+                        for (int c = 0; c < kMaxCover; ++c) {
+                            if (c < nj) {
+                                const int k = i * cols + jhi - c;
+                                const float4 f = __ldcs(reinterpret_cast<const float4*>(
+                                    field + (size_t)k * L * L + (size_t)(Y - sy) * L + (X - sxs[c])));
+                                const float2 zk = z[k];
+                                const float w0 = wy * wxa[c], w1 = wy * wxb[c];
+                                ar0 += w0 * (f.x * zk.x - f.y * zk.y);
+                                ai0 += w0 * (f.x * zk.y + f.y * zk.x);
+                                ws0 += w0;
+                                ar1 += w1 * (f.z * zk.x - f.w * zk.y);
+                                ai1 += w1 * (f.z * zk.y + f.w * zk.x);
+                                ws1 += w1;
+                            }
                         }
                     }
                 }
+                o = make_float4(ws0 > 0.f ? ar0 / ws0 : 0.f, ws0 > 0.f ? ai0 / ws0 : 0.f,
+                                ws1 > 0.f ? ar1 / ws1 : 0.f, ws1 > 0.f ? ai1 / ws1 : 0.f);
             }
-            o = make_float4(ws0 > 0.f ? ar0 / ws0 : 0.f, ws0 > 0.f ? ai0 / ws0 : 0.f,
-                            ws1 > 0.f ? ar1 / ws1 : 0.f, ws1 > 0.f ? ai1 / ws1 : 0.f);
+            __stcs(reinterpret_cast<float4*>(out + (size_t)Y * Wo + X), o);
         }
-        __stcs(reinterpret_cast<float4*>(out + (size_t)Y * Wo + X), o);
     }
 }
 
