@@ -59,7 +59,6 @@ k_kk_reg(DevPlan P, int n_tiles, const float* __restrict__ I, float2* __restrict
     const T4Lane L(t);
     const int lrow = t4_row(t, n), lcol = t4_col(t);      // this lane's row / column offsets
     const float inv_n2 = 1.0f / (float)(n * n);
-    const long long hh = (long long)P.h * P.h, ww = (long long)P.w * P.w;
     const int nprob = n_tiles * P.n_bf;
 
     int par = 0;
@@ -102,13 +101,13 @@ k_kk_reg(DevPlan P, int n_tiles, const float* __restrict__ I, float2* __restrict
 #pragma unroll
             for (int j = 0; j < BN; ++j) v[j] = gc[16 * j * n];
             fft_a<BN, false>(v, o, h, tw);
-            const long long kxp = (long long)sfreq_kk(x, n) * kix * hh;
+            const int kxp = sfreq_kk(x, n) * kix;             // square tiles: k . k_i up to a common factor
 #pragma unroll
             for (int s = 0; s < S; ++s)
                 if (t + 16 * s < BN) {
 #pragma unroll
                     for (int k1 = 0; k1 < 16; ++k1) {
-                        const long long dot = kxp + (long long)sfreq_kk(t + 16 * s + BN * k1, n) * kiy * ww;
+                        const int dot = kxp + sfreq_kk(t + 16 * s + BN * k1, n) * kiy;
                         const float f = dot < 0 ? 1.f : (dot == 0 ? 0.5f : 0.f);
                         o[s][k1] = cscale(o[s][k1], f);
                     }
