@@ -1,0 +1,50 @@
+// cluster.cuh - set-up and launch of kernels that run on clusters of K blocks (K = 1: plain blocks).
+#pragma once
+
+#include "common.cuh"
+
+namespace apic {
+
+inline void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, int K, int slots, int threads,
+                           size_t smem, cudaStream_t st) {
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = K;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(K * slots, 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = K > 1 ? 1 : 0;
+}
+
+// Blocks (K = 1) or clusters of K blocks of kernel f that run at once on the current
+// device, 0 on error; raises the kernel's shared-memory limit.
+inline int cluster_slots(const void* f, int threads, size_t smem, int K) {
+    if (!f || raise_smem_limit(f, smem) != cudaSuccess) return 0;
+    if (K == 1) {
+        int occ = 0, dev = 0, sms = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, threads, smem) != cudaSuccess ||
+            cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return 0;
+        return occ * sms;
+    }
+    if (K > 8 && cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return 0;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr;
+    cluster_config(cfg, attr, K, 256, threads, smem, nullptr);
+    int clusters = 0;
+    return cudaOccupancyMaxActiveClusters(&clusters, f, &cfg) == cudaSuccess ? clusters : 0;
+}
+
+template <class... P, class... A>
+cudaError_t cluster_launch(void (*f)(P...), int K, int slots, int threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr;
+    cluster_config(cfg, attr, K, slots, threads, smem, st);
+    return cudaLaunchKernelEx(&cfg, f, args...);
+}
+
+}  // namespace apic

@@ -6,12 +6,14 @@
 
 // Complex adds and subtracts as packed FP32 pairs (add.f32x2: one issue slot for both
 // parts, the same rounding and the same 128 lanes per cycle and SM) in the translation
-// units that define APIC_PACKED_ADDS, the darkfield kernels: half the issue slots of
-// their transforms' additions took 7 % off a wave of 256- or 512-pixel tiles (65.5 ->
-// 61.2 ms for 512 tiles of 256). The Kramers-Kronig stage keeps scalar adds: the packed
-// form stops some multiply-adds from being fused, and a last-bit change of a recovered
-// phase can wrap a row of the aberration system (Eq. 10) the other way. The two flavours
-// live in inline namespaces of their own, so that no function has two definitions.
+// unit that defines APIC_PACKED_ADDS, the darkfield kernel of 512-pixel tiles: half the
+// issue slots of its transforms' additions, 400 tiles 270 -> 250 ms. The packed form keeps
+// some multiply-adds from being fused, so the other units keep scalar adds: a last-bit
+// change of a Kramers-Kronig phase can wrap a row of the aberration system (Eq. 10) the
+// other way, and the darkfield solves of smaller tiles serve slides whose windows may hold
+// seams: ill-conditioned solves, whose last iterate depends on the last bit of every sum
+// (there the packed form moved a field by 3e-4). The two flavours live in inline
+// namespaces of their own, so that no function has two definitions.
 #ifdef APIC_PACKED_ADDS
 #define APIC_ARITH packed_adds
 #else
@@ -113,6 +115,31 @@ __device__ __forceinline__ double block_sum2f(float v, double* red, int& parity)
     }
     __syncthreads();
     const double total = r[31];
+    parity ^= 1;
+    return total;
+}
+
+// block_sum2f with a quotient of the sum, rounded to FP32: num / sum, or (OVER) sum / num.
+// One thread divides: an FP64 division by every warp costs about as much pipe time as a
+// pass over the rows of unknowns.
+template <bool OVER>
+__device__ __forceinline__ double block_sum2f_ratio(float v, double num, double* red, int& parity, float& ratio) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+    double* r = red + parity * 32;
+    if (lane == 0) r[warp] = (double)v;
+    __syncthreads();
+    if (warp == 0) {
+        double t = lane < nw ? r[lane] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) {
+            r[31] = t;
+            r[30] = OVER ? t / num : num / t;
+        }
+    }
+    __syncthreads();
+    const double total = r[31];
+    ratio = (float)r[30];
     parity ^= 1;
     return total;
 }

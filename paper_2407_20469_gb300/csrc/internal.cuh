@@ -36,6 +36,7 @@ struct DevPlan {
     int qmask_words;                 // Q membership words per band row (8; 16 for the wide kernel)
     int max_mx, max_mxy;             // wide kernel: largest row grid and row x column grid of the used images
     int band_u, band_p, band_q;      // largest U, P and Q row bands of the used images
+    int cl_mx, cl_maxB;              // largest row grid, and row or column grid / 16, of the used images
     int max_N, max_M;
     float Rx, Ry;
     int pup_ax, pup_ay;
@@ -153,10 +154,20 @@ cudaError_t launch_darkfield_reg(const DevPlan& P, int grid, size_t smem, int n_
                                  float tol, int32_t* status, unsigned long long* counters, int* work,
                                  cudaStream_t st);
 
+// cluster darkfield kernel of 128- and 256-pixel tiles (dfc.cuh): K blocks per tile, the band
+// grids in their shared memory. configure_dfc returns the clusters that run at once for the
+// plan's current tables (0: not available); scratch holds dfc_scratch_bytes per cluster.
+constexpr int kMaxCluster = 16;
+int configure_dfc(const DevPlan& P, int K);
+size_t dfc_scratch_bytes(const DevPlan& P);
+cudaError_t launch_darkfield_cluster(const DevPlan& P, int K, int slots, int n_tiles, const float* I, const float* phi,
+                                     float2* spec, void* scratch, int iters, float tol, int32_t* status,
+                                     unsigned long long* counters, cudaStream_t st);
+
 // wide darkfield kernel of 512-pixel tiles (kernels_dfw.cu)
 size_t dfw_smem_bytes(int max_N, int band);   // band: max of the U, P and Q row bands
 size_t dfw_scratch_bytes(const DevPlan& P);
-// tile slots (clusters of K blocks, K in 1, 2, 4) that run at once; grid = tile slots
+// tile slots (clusters of K <= kMaxCluster blocks) that run at once; grid = tile slots
 int configure_dfw(size_t smem, int K);
 cudaError_t launch_darkfield_wide(const DevPlan& P, int K, int grid, size_t smem, int n_tiles, const float* I,
                                   const float* phi, float2* spec, void* scratch, size_t per_block, int iters,

@@ -28,15 +28,18 @@
 // every block takes the same steps. With K blocks per tile only 1/K as many tiles are
 // in flight, so their band grids stay in L2 instead of going to HBM. Data another
 // block wrote is read with L2-only loads (no stale L1 lines).
-// Transforms, vectors and per-thread / per-warp partial sums FP32; the sums across
-// warps and blocks and the CG step lengths FP64.
+// Transforms, vectors and the sums within a row FP32; the sums across rows as float pairs
+// (about 48 bits).
+#define APIC_PACKED_ADDS 1
 #include <math.h>
 
 #include <algorithm>
 
 #include "../../include/apic.h"
+#include "cluster.cuh"
 #include "internal.cuh"
 #include "regfft.cuh"
+#include "rowsum.cuh"
 #include "t4grid.cuh"
 
 namespace apic {
@@ -70,11 +73,17 @@ __device__ __forceinline__ unsigned cta_rank() {
     return r;
 }
 
+__device__ __forceinline__ unsigned cta_count() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+
 // Barrier of all threads of the K blocks of a tile (release / acquire at cluster
 // scope); a block barrier when K = 1.
-template <int K>
+template <bool CL>
 __device__ __forceinline__ void tile_sync() {
-    if constexpr (K == 1) {
+    if constexpr (!CL) {
         __syncthreads();
     } else {
         asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -82,51 +91,34 @@ __device__ __forceinline__ void tile_sync() {
 }
 
 // Load of scratch data that another block of the cluster may have written: from L2.
-template <int K>
+template <bool CL>
 __device__ __forceinline__ float2 ldx(const float2* p) {
-    if constexpr (K == 1)
+    if constexpr (!CL)
         return *p;
     else
         return __ldcg(p);
 }
 
-// Sum over the tile's K blocks of FP32 per-thread values: FP32 within warps, FP64
-// across the block's warps (warp 0) and across the blocks (each block's total stored
-// into slot `rank` of every block's area through distributed shared memory, then
-// summed in rank order, so all blocks hold the same value). red: 96 doubles;
-// `parity` alternates so that a slot is never rewritten while a block still reads it.
-template <int K>
-__device__ __forceinline__ double tile_sum(float v, double* red, int& parity) {
-    if constexpr (K == 1) {
-        return block_sum2f(v, red, parity);
-    } else {
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-        double* r = red + parity * 32;
-        double* slots = red + 64 + parity * 16;
-        if (lane == 0) r[warp] = (double)v;
-        __syncthreads();
-        if (warp == 0) {
-            double t = lane < nw ? r[lane] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane < K) {          // lane q stores this block's total into block q's slot
-                const unsigned a = (unsigned)__cvta_generic_to_shared(slots + cta_rank());
-                unsigned ra;
-                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"((unsigned)lane));
-                asm volatile("st.shared::cluster.f64 [%0], %1;" :: "r"(ra), "d"(t) : "memory");
-            }
-        }
-        tile_sync<K>();
-        double total = 0.0;
+// The sum of a U row's values over the half-warp, into entry b of the list rs of every
+// block of the tile (its own through distributed shared memory as well).
+template <bool CL>
+__device__ __forceinline__ void wrow_sum(const HWw& w, float v, int b, float* rs) {
 #pragma unroll
-        for (int q = 0; q < K; ++q) total += slots[q];
-        parity ^= 1;
-        return total;
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(w.mask, v, o, 16);
+    if constexpr (!CL) {
+        if (w.t == 0) rs[b] = v;
+    } else {
+        if (w.t < w.ghs / kWHW) {
+            const unsigned a = (unsigned)__cvta_generic_to_shared(rs + b);
+            unsigned ra;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"((unsigned)w.t));
+            asm volatile("st.shared::cluster.f32 [%0], %1;" :: "r"(ra), "f"(v) : "memory");
+        }
     }
 }
 
 // ---- per-point functors (as in the 256-pixel kernel)
-template <int K>
+template <bool CL>
 struct WValKnown {      // P(c) = O_known(K) exp(j phi(c)) (the spectrum: written by any block of the tile)
     const float2* sp;
     const float* ph;
@@ -135,7 +127,7 @@ struct WValKnown {      // P(c) = O_known(K) exp(j phi(c)) (the spectrum: writte
     __device__ float2 operator()(int e) const {
         float sn, cs;
         sincosf(ph[pup[e]], &sn, &cs);
-        return cmul(ldx<K>(sp + ap[e]), make_float2(cs, sn));
+        return cmul(ldx<CL>(sp + ap[e]), make_float2(cs, sn));
     }
 };
 struct WValNextDir {    // d = s + beta d (stored back)
@@ -265,20 +257,19 @@ __device__ __noinline__ void wpass_rows_in(HWw w, const float2* tw, float2* G, i
     }
 }
 
-// rows of a band of the tiled grid G (ld columns): forward transform along x; returns
-// the sum of out(e, value) over this lane's points.
-template <int B, int K, class Out>
-__device__ __noinline__ float wpass_rows_out(HWw w, const float2* tw, const float2* G, int ld, int nrows,
-                                             const int* rp, const int* px, Out out) {
+// rows of a band of the tiled grid G (ld columns): forward transform along x; the sum of
+// out(e, value) over each row into the list rs.
+template <int B, bool CL, class Out>
+__device__ __noinline__ void wpass_rows_out(HWw w, const float2* tw, const float2* G, int ld, int nrows,
+                                            const int* rp, const int* px, Out out, float* rs) {
     constexpr int m = 16 * B, S = Slots<B>::value;
     const HalfWarp h = w.h();
-    float acc = 0.f;
     const int c0 = t4_col(w.t);
     for (int b = w.gh; b < nrows; b += w.ghs) {
         const float2* row = G + t4_row(b, ld) + c0;
         float2 v[B], o[S][16];
 #pragma unroll
-        for (int j = 0; j < B; ++j) v[j] = ldx<K>(row + 64 * j);
+        for (int j = 0; j < B; ++j) v[j] = ldx<CL>(row + 64 * j);
         // the row's point range and this lane's first point, loaded before the transform
         const int e0 = rp[b] + w.t, e1 = rp[b + 1];
         int xn = e0 < e1 ? px[e0] : 0;
@@ -290,14 +281,15 @@ __device__ __noinline__ float wpass_rows_out(HWw w, const float2* tw, const floa
                 for (int k1 = 0; k1 < 16; ++k1) w.hs[w.t + 16 * s + B * k1] = o[s][k1];
             }
         __syncwarp(w.mask);
+        float acc = 0.f;
         for (int e = e0; e < e1; e += 16) {
             const int xc = xn;
             if (e + 16 < e1) xn = px[e + 16];
             acc += out(e, w.hs[freq_index(xc, m)]);
         }
         __syncwarp(w.mask);
+        wrow_sum<CL>(w, acc, b, rs);
     }
-    return acc;
 }
 
 // columns x < ncols of a grid whose columns have 16 B points: the ni band rows of the
@@ -316,7 +308,7 @@ __device__ __noinline__ float wpass_rows_out(HWw w, const float2* tw, const floa
 // transform; both slowed the kernel by ~10 %: the first adds block barriers between
 // half-warps that otherwise overlap one another's loads and transforms, the second
 // spills.)
-template <int B, int K, class Mid>
+template <int B, bool CL, class Mid>
 __device__ __noinline__ void wpass_cols(HWw w, const float2* tw, int ncols, const float2* Gi, int ldi, int ni,
                                         float2* Go, int ldo, int no, Mid mid) {
     constexpr int S = Slots<B>::value;
@@ -327,7 +319,7 @@ __device__ __noinline__ void wpass_cols(HWw w, const float2* tw, int ncols, cons
         const float2* gi = Gi + ri + t4_col(x);
 #pragma unroll
         for (int j = 0; j < B; ++j)                                  // band row t + 16 j
-            v[j] = w.t + 16 * j < ni ? ldx<K>(gi + 16 * j * ldi) : make_float2(0.f, 0.f);
+            v[j] = w.t + 16 * j < ni ? ldx<CL>(gi + 16 * j * ldi) : make_float2(0.f, 0.f);
         if constexpr (Mid::kPre) {
             typename Mid::Pre pre;
             mid.load(pre, x, w.t);
@@ -345,13 +337,13 @@ __device__ __noinline__ void wpass_cols(HWw w, const float2* tw, int ncols, cons
                 if (w.t + 16 * k1 < no) go[16 * k1 * ldo] = v[k1];
         }
     }
-    tile_sync<K>();
+    tile_sync<CL>();
 }
 
 // rows of Q in place (tiled grid of 16 B columns): forward along x, keep the Q lags, inverse
 // along x. qmask: per band row 16 words; the bit k1 of half (t + 16 s) & 1 of word
 // (t + 16 s) >> 1 says whether x index (t + 16 s) + B k1 is in Q. Ends with __syncthreads.
-template <int B, int K>
+template <int B, bool CL>
 __device__ __noinline__ void wpass_rows_mask(HWw w, const float2* tw, float2* G, int nrows, const unsigned* qmask) {
     constexpr int m = 16 * B, S = Slots<B>::value;
     const HalfWarp h = w.h();
@@ -360,7 +352,7 @@ __device__ __noinline__ void wpass_rows_mask(HWw w, const float2* tw, float2* G,
         float2* row = G + t4_row(b, m) + c0;
         float2 v[B], o[S][16];
 #pragma unroll
-        for (int j = 0; j < B; ++j) v[j] = ldx<K>(row + 64 * j);
+        for (int j = 0; j < B; ++j) v[j] = ldx<CL>(row + 64 * j);
         unsigned qw[S];
 #pragma unroll
         for (int s = 0; s < S; ++s) qw[s] = qmask[(size_t)b * kWQWords + ((w.t + 16 * s) >> 1)];
@@ -377,7 +369,7 @@ __device__ __noinline__ void wpass_rows_mask(HWw w, const float2* tw, float2* G,
 #pragma unroll
         for (int k1 = 0; k1 < B; ++k1) row[64 * k1] = v[k1];
     }
-    tile_sync<K>();
+    tile_sync<CL>();
 }
 
 // Columns of I - |p|^2 (n = 512; the image read transposed with tr, once, with
@@ -389,14 +381,14 @@ __device__ __noinline__ void wpass_rows_mask(HWw w, const float2* tw, float2* G,
 // formed and transformed forward along y; rows qy0.. (nQ) go to GX (row length n).
 // Half-warps 0..31 take one column of a chunk each. The stages alias the half-warp
 // areas; barriers separate each use from the transforms. Ends with a tile barrier.
-template <int K>
+template <bool CL>
 __device__ __noinline__ void wpass_image_cols_p(HWw w, const float2* tw, float2* stage, const float* img,
                                                 const float2* GP, int nP, float2* GX, int qy0, int nQ,
                                                 bool tr) {
     constexpr int BN = kWBN, n = 16 * BN, S = Slots<BN>::value;
     const HalfWarp h = w.h();
     float* stage_f = reinterpret_cast<float*>(stage);
-    for (int c0 = 32 * (w.gh / kWHW); c0 < n; c0 += 32 * K) {     // this block's chunks of 32 columns
+    for (int c0 = 32 * (w.gh / kWHW); c0 < n; c0 += 32 * (w.ghs / kWHW)) {     // this block's chunks of 32 columns
         const int x = c0 + w.hw;
         float2 v[BN], o[S][16];
         float q[S][16];
@@ -404,7 +396,7 @@ __device__ __noinline__ void wpass_image_cols_p(HWw w, const float2* tw, float2*
         // y, which |p|^2 does not see
         const float2* gp = GP + t4_row(w.t, n) + t4_col(x);
 #pragma unroll
-        for (int j = 0; j < BN; ++j) v[j] = w.t + 16 * j < nP ? ldx<K>(gp + 16 * j * n) : make_float2(0.f, 0.f);
+        for (int j = 0; j < BN; ++j) v[j] = w.t + 16 * j < nP ? ldx<CL>(gp + 16 * j * n) : make_float2(0.f, 0.f);
         fft_a<BN, true>(v, o, h, tw);               // p(x, y), y = (t + 16 s) + BN k1
 #pragma unroll
         for (int s = 0; s < S; ++s)
@@ -445,12 +437,12 @@ __device__ __noinline__ void wpass_image_cols_p(HWw w, const float2* tw, float2*
         }
         __syncthreads();
     }
-    tile_sync<K>();
+    tile_sync<CL>();
 }
 
 // rows of GX (length n): forward along x, bq[e] = value / n^2 at the Q points. Ends
 // with __syncthreads.
-template <int K>
+template <bool CL>
 __device__ __noinline__ void wpass_image_rows(HWw w, const float2* tw, const float2* GX, int nQ, const int* qrp,
                                               const int* Qx, float2* bq) {
     constexpr int BN = kWBN, n = 16 * BN, S = Slots<BN>::value;
@@ -460,7 +452,7 @@ __device__ __noinline__ void wpass_image_rows(HWw w, const float2* tw, const flo
         const float2* row = GX + (size_t)b * n;
         float2 v[BN], o[S][16];
 #pragma unroll
-        for (int j = 0; j < BN; ++j) v[j] = ldx<K>(row + w.t + 16 * j);
+        for (int j = 0; j < BN; ++j) v[j] = ldx<CL>(row + w.t + 16 * j);
         fft_a<BN, false>(v, o, h, tw);
 #pragma unroll
         for (int s = 0; s < S; ++s)
@@ -472,7 +464,7 @@ __device__ __noinline__ void wpass_image_rows(HWw w, const float2* tw, const flo
         for (int e = qrp[b] + w.t; e < qrp[b + 1]; e += 16) bq[e] = cscale(w.hs[freq_index(Qx[e], n)], inv_n2);
         __syncwarp(w.mask);
     }
-    tile_sync<K>();
+    tile_sync<CL>();
 }
 
 }  // namespace
@@ -485,7 +477,7 @@ __device__ __noinline__ void wpass_image_rows(HWw w, const float2* tw, const flo
 //                     stage, or the output stage of the image columns
 //   [tw, tw_end)      step twiddles of the camera grid and of the image's row and
 //                     column grids
-//   [red, total)      96 doubles of reductions (block partials, then the blocks' totals)
+//   [red, total)      two lists of the U rows' sums
 struct DFWSmem {
     size_t vec, tw, red, total;
 };
@@ -503,7 +495,7 @@ __host__ __device__ inline DFWSmem dfw_smem_layout(int max_N, int band) {
     const size_t setup = std::max(setup_hw, std::max(stage_c, stage_f));
     L.tw = walign16(std::max(cg_end, setup));
     L.red = walign16(L.tw + (size_t)2 * 16 * (kWBN + 2 * kWMaxB) * sizeof(float2));
-    L.total = walign16(L.red + 96 * sizeof(double));
+    L.total = walign16(L.red + (size_t)2 * band * sizeof(float));
     return L;
 }
 
@@ -532,7 +524,8 @@ struct DFWCtx {
     float2 *GU, *GQ, *PF, *bq;
     float2 *dv, *sv, *wv, *xv;
     float2* stage;          // stages of the setup column pass (alias the half-warp areas)
-    double* red;
+    float* rs;              // two lists of the U rows' sums, n_rs entries each
+    int n_rs;
 };
 
 // plain twiddle table of a 16 G-point grid of the wide solve
@@ -543,7 +536,7 @@ __device__ __forceinline__ const float2* wgrid_table(const DevPlan& P, int G) {
 // Solve of one darkfield image (image `img`) on a grid of 16 BX row points x 16 BY
 // column points, by the K blocks of the cluster: b = F(I - |p|^2) on Q on the camera
 // grid, then CGNR. Returns the CG iterations (negative: did not converge).
-template <int BX, int BY, int K>
+template <int BX, int BY, bool CL>
 __device__ __forceinline__ int dfw_solve(const DFWCtx& c, const DevPlan& P, const DevDF& D, const float* img,
                                          float2* sp, const float* ph, int iters, float tol) {
     constexpr int n = 16 * kWBN, mx = 16 * BX;
@@ -553,7 +546,7 @@ __device__ __forceinline__ int dfw_solve(const DFWCtx& c, const DevPlan& P, cons
     const int nU = D.uy1 - uy0 + 1, nQ = D.qy1 - qy0 + 1, nP = D.py1 - py0 + 1;
     const int *urp = P.d_rowptr + D.urp, *qrp = P.d_rowptr + D.qrp, *prp = P.d_rowptr + D.prp;
     const unsigned* qmask = P.d_qmask + D.qmask_off;
-    const WValKnown<K> pval{sp, ph, P.dP_ap + p_off, P.dP_pup + p_off};
+    const WValKnown<CL> pval{sp, ph, P.dP_ap + p_off, P.dP_pup + p_off};
     make_step_twiddles(c.tw_x, wgrid_table(P, BX), BX);
     make_step_twiddles(c.tw_y, wgrid_table(P, BY), BY);
     __syncthreads();
@@ -561,66 +554,63 @@ __device__ __forceinline__ int dfw_solve(const DFWCtx& c, const DevPlan& P, cons
     // (exact: P * P's lags reach 2 R < n / 2): the known field's band rows along x,
     // then per column p, the difference and its forward transform, then the rows
     wpass_rows_in<kWBN>(c.ws, c.tw_n, c.GQ, n, nP, prp, P.dP_x + p_off, pval);
-    tile_sync<K>();
-    wpass_image_cols_p<K>(c.ws, c.tw_n, c.stage, img, c.GQ, nP, c.PF, qy0, nQ, D.tr != 0);
-    wpass_image_rows<K>(c.ws, c.tw_n, c.PF, nQ, qrp, P.dQ_x + q_off, c.bq);
+    tile_sync<CL>();
+    wpass_image_cols_p<CL>(c.ws, c.tw_n, c.stage, img, c.GQ, nP, c.PF, qy0, nQ, D.tr != 0);
+    wpass_image_rows<CL>(c.ws, c.tw_n, c.PF, nQ, qrp, P.dQ_x + q_off, c.bq);
     // band rows of the known field P (Eq. 11) along x on the row grid, then p s on
     // the column grid, column-major in PF (s = 1 / (mx my): the two unnormalised
     // transforms around each product)
     const float scale = 1.f / ((float)mx * (float)(16 * BY));
     wpass_rows_in<BX>(w, c.tw_x, c.GQ, mx, nP, prp, P.dP_x + p_off, pval);
-    tile_sync<K>();
+    tile_sync<CL>();
     // the field carries the ramp W^((uy0 - qy0) k) of the U <-> Q column passes and
     // W^(-py0 k) for its own band's start (see wpass_cols)
     const int my = 16 * BY, shift = (((uy0 - qy0 - py0) % my) + my) % my;
-    wpass_cols<BY, K>(w, c.tw_y, mx, c.GQ, mx, nP, c.GQ, mx, 0,
+    wpass_cols<BY, CL>(w, c.tw_y, mx, c.GQ, mx, nP, c.GQ, mx, 0,
                       WMidStoreField<BY>{c.PF, scale, wgrid_table(P, BY), shift});
     // rows of b inverse along x on the row grid; s = d = C^H b
     wpass_rows_in<BX>(w, c.tw_x, c.GQ, mx, nQ, qrp, P.dQ_x + q_off, WValB{c.bq});
-    tile_sync<K>();
-    wpass_cols<BY, K>(w, c.tw_y, mx, c.GQ, mx, nQ, c.GU, mx, nU, WMidTimesField<BY, false>{c.PF});
-    const float g0 =
-        wpass_rows_out<BX, K>(w, c.tw_x, c.GU, mx, nU, urp, P.dU_x + u_off, WOutStart{c.sv, c.dv, c.xv});
-    int par = 0;
-    const double gamma0 = tile_sum<K>(g0, c.red, par);
-    // CGNR; each block updates the vector entries of its own U rows
-    double gamma = gamma0;
-    bool conv = !(gamma0 > 1e-300);
-    const double stop = (double)tol * (double)tol * gamma0;
+    tile_sync<CL>();
+    wpass_cols<BY, CL>(w, c.tw_y, mx, c.GQ, mx, nQ, c.GU, mx, nU, WMidTimesField<BY, false>{c.PF});
+    wpass_rows_out<BX, CL>(w, c.tw_x, c.GU, mx, nU, urp, P.dU_x + u_off, WOutStart{c.sv, c.dv, c.xv}, c.rs);
+    tile_sync<CL>();
+    // CGNR; each half-warp updates the vector entries of the U rows it gathered. Every warp
+    // forms the scalars itself, from the same sums in the same order.
+    FF gamma = row_total(c.rs, nU);
+    const CgStop stop(tol, gamma.hi);
+    bool conv = !(gamma.hi > 0.f);
     int it = 0;
     float bf = 0.f;
     for (; it < iters && !conv; ++it) {
         wpass_rows_in<BX>(w, c.tw_x, c.GU, mx, nU, urp, P.dU_x + u_off, WValNextDir{c.sv, c.dv, bf});
-        tile_sync<K>();
-        wpass_cols<BY, K>(w, c.tw_y, mx, c.GU, mx, nU, c.GQ, mx, nQ, WMidTimesField<BY, true>{c.PF});
-        wpass_rows_mask<BX, K>(w, c.tw_x, c.GQ, nQ, qmask);
-        wpass_cols<BY, K>(w, c.tw_y, mx, c.GQ, mx, nQ, c.GU, mx, nU, WMidTimesField<BY, false>{c.PF});
-        const float dw = wpass_rows_out<BX, K>(w, c.tw_x, c.GU, mx, nU, urp, P.dU_x + u_off, WOutDot{c.wv, c.dv});
-        const double delta = tile_sum<K>(dw, c.red, par);
-        if (!(delta > 0)) break;
-        const double alpha = gamma / delta;
-        const float af = (float)alpha;
-        float g2 = 0.f;
-        auto update = [&](int e) {
-            const float2 d = c.dv[e];
-            float2 x = c.xv[e];
-            x.x += af * d.x;
-            x.y += af * d.y;
-            c.xv[e] = x;
-            const float2 sv = csub(c.sv[e], cscale(c.wv[e], af));
-            c.sv[e] = sv;
-            g2 += sv.x * sv.x + sv.y * sv.y;
-        };
-        if constexpr (K == 1) {           // all entries are this block's: every thread an even share
-            for (int e = threadIdx.x; e < D.N; e += blockDim.x) update(e);
-        } else {                          // the entries of this block's U rows
-            for (int b = w.gh; b < nU; b += w.ghs)
-                for (int e = urp[b] + w.t; e < urp[b + 1]; e += 16) update(e);
+        tile_sync<CL>();
+        wpass_cols<BY, CL>(w, c.tw_y, mx, c.GU, mx, nU, c.GQ, mx, nQ, WMidTimesField<BY, true>{c.PF});
+        wpass_rows_mask<BX, CL>(w, c.tw_x, c.GQ, nQ, qmask);
+        wpass_cols<BY, CL>(w, c.tw_y, mx, c.GQ, mx, nQ, c.GU, mx, nU, WMidTimesField<BY, false>{c.PF});
+        wpass_rows_out<BX, CL>(w, c.tw_x, c.GU, mx, nU, urp, P.dU_x + u_off, WOutDot{c.wv, c.dv}, c.rs);
+        tile_sync<CL>();
+        const FF delta = row_total(c.rs, nU);
+        if (!(delta.hi > 0.f)) break;
+        const float af = ff_div(gamma, delta);
+        for (int b = w.gh; b < nU; b += w.ghs) {
+            float g2 = 0.f;
+            for (int e = urp[b] + w.t; e < urp[b + 1]; e += 16) {
+                const float2 d = c.dv[e];
+                float2 x = c.xv[e];
+                x.x += af * d.x;
+                x.y += af * d.y;
+                c.xv[e] = x;
+                const float2 sv = csub(c.sv[e], cscale(c.wv[e], af));
+                c.sv[e] = sv;
+                g2 += sv.x * sv.x + sv.y * sv.y;
+            }
+            wrow_sum<CL>(w, g2, b, c.rs + c.n_rs);
         }
-        const double gnew = tile_sum<K>(g2, c.red, par);
-        bf = (float)(gnew / gamma);
+        tile_sync<CL>();
+        const FF gnew = row_total(c.rs + c.n_rs, nU);
+        bf = ff_div(gnew, gamma);
+        conv = stop.reached(gnew.hi);
         gamma = gnew;
-        conv = gnew <= stop;
     }
     // corrected unknown spectrum into the tile's spectrum (this block's U rows)
     const int* Upup = P.dU_pup + u_off;
@@ -630,17 +620,13 @@ __device__ __forceinline__ int dfw_solve(const DFWCtx& c, const DevPlan& P, cons
         sincosf(ph[Upup[e]], &sn, &cs);
         sp[Uap[e]] = cmul(c.xv[e], make_float2(cs, -sn));
     };
-    if constexpr (K == 1) {
-        for (int e = threadIdx.x; e < D.N; e += blockDim.x) put(e);
-    } else {
-        for (int b = w.gh; b < nU; b += w.ghs)
-            for (int e = urp[b] + w.t; e < urp[b + 1]; e += 16) put(e);
-    }
-    tile_sync<K>();
+    for (int b = w.gh; b < nU; b += w.ghs)
+        for (int e = urp[b] + w.t; e < urp[b + 1]; e += 16) put(e);
+    tile_sync<CL>();
     return conv ? it : -1 - it;
 }
 
-template <int K>
+template <bool CL>
 __global__ void __launch_bounds__(kWThreads, 1)
 k_darkfield_wide(DevPlan P, int n_tiles, const float* __restrict__ I, const float* __restrict__ phi,
                  float2* __restrict__ spec, char* __restrict__ scratch, size_t per_block, int iters, float tol,
@@ -659,10 +645,11 @@ k_darkfield_wide(DevPlan P, int n_tiles, const float* __restrict__ I, const floa
     c.tw_n = tw_n;
     c.tw_x = tw_n + 2 * 16 * kWBN;
     c.tw_y = c.tw_x + 2 * 16 * kWMaxB;
-    c.red = reinterpret_cast<double*>(sbase + SL.red);
+    c.rs = reinterpret_cast<float*>(sbase + SL.red);
+    c.n_rs = P.band_u;
     make_step_twiddles(tw_n, P.tw_n, kWBN);
 
-    const int rank = K > 1 ? (int)cta_rank() : 0;
+    const int rank = CL ? (int)cta_rank() : 0, K = CL ? (int)cta_count() : 1;
     const int slot = blockIdx.x / K, nslots = gridDim.x / K;      // tile slot = the cluster
     c.w.hw = c.ws.hw = threadIdx.x >> 4;
     c.w.gh = c.ws.gh = rank * kWHW + c.w.hw;
@@ -677,14 +664,14 @@ k_darkfield_wide(DevPlan P, int n_tiles, const float* __restrict__ I, const floa
     c.PF = c.GQ + (size_t)t4_rows(max(P.band_q, P.band_p)) * n;
     c.GU = c.PF + max((size_t)P.max_mxy, (size_t)P.band_q * n);
     c.bq = c.GU + (size_t)t4_rows(P.band_u) * P.max_mx;
-    tile_sync<K>();
+    tile_sync<CL>();
 
     // one block per tile: tiles taken one at a time from the launch's counter (a block that
     // meets skipped background tiles goes on to the next, so uneven batches balance);
     // clusters (and launches without a counter): by stride
     __shared__ int s_next;
     auto take = [&](int prev) -> int {
-        if (K > 1 || !work) return prev < 0 ? slot : prev + nslots;
+        if (CL || !work) return prev < 0 ? slot : prev + nslots;
         __syncthreads();
         if (threadIdx.x == 0) s_next = atomicAdd(work, 1);
         __syncthreads();
@@ -700,13 +687,13 @@ k_darkfield_wide(DevPlan P, int n_tiles, const float* __restrict__ I, const floa
             const float* img = I + ((size_t)tile * P.n_img + D.led) * n * n;
             int r;
             switch (16 * D.bx + D.by) {
-                case 16 * 18 + 12: r = dfw_solve<18, 12, K>(c, P, D, img, sp, ph, iters, tol); break;
-                case 16 * 18 + 16: r = dfw_solve<18, 16, K>(c, P, D, img, sp, ph, iters, tol); break;
-                case 16 * 18 + 18: r = dfw_solve<18, 18, K>(c, P, D, img, sp, ph, iters, tol); break;
-                case 16 * 20 + 12: r = dfw_solve<20, 12, K>(c, P, D, img, sp, ph, iters, tol); break;
-                case 16 * 20 + 16: r = dfw_solve<20, 16, K>(c, P, D, img, sp, ph, iters, tol); break;
-                case 16 * 20 + 18: r = dfw_solve<20, 18, K>(c, P, D, img, sp, ph, iters, tol); break;
-                default: r = dfw_solve<20, 20, K>(c, P, D, img, sp, ph, iters, tol); break;
+                case 16 * 18 + 12: r = dfw_solve<18, 12, CL>(c, P, D, img, sp, ph, iters, tol); break;
+                case 16 * 18 + 16: r = dfw_solve<18, 16, CL>(c, P, D, img, sp, ph, iters, tol); break;
+                case 16 * 18 + 18: r = dfw_solve<18, 18, CL>(c, P, D, img, sp, ph, iters, tol); break;
+                case 16 * 20 + 12: r = dfw_solve<20, 12, CL>(c, P, D, img, sp, ph, iters, tol); break;
+                case 16 * 20 + 16: r = dfw_solve<20, 16, CL>(c, P, D, img, sp, ph, iters, tol); break;
+                case 16 * 20 + 18: r = dfw_solve<20, 18, CL>(c, P, D, img, sp, ph, iters, tol); break;
+                default: r = dfw_solve<20, 20, CL>(c, P, D, img, sp, ph, iters, tol); break;
             }
             if (r < 0) notconv = true;
             if (threadIdx.x == 0 && rank == 0 && counters) {
@@ -725,41 +712,11 @@ using DFWKernel = void (*)(DevPlan, int, const float*, const float*, float2*, ch
                            unsigned long long*, int*);
 
 static DFWKernel dfw_kernel(int K) {
-    switch (K) {
-        case 1: return k_darkfield_wide<1>;
-        case 2: return k_darkfield_wide<2>;
-        case 4: return k_darkfield_wide<4>;
-        default: return nullptr;
-    }
+    return K == 1 ? k_darkfield_wide<false> : K >= 2 && K <= kMaxCluster ? k_darkfield_wide<true> : nullptr;
 }
 
 // Tile slots (clusters of K blocks) that run at once, 0 on error.
-int configure_dfw(size_t smem, int K) {
-    DFWKernel f = dfw_kernel(K);
-    if (!f || raise_smem_limit((const void*)f, smem) != cudaSuccess) return 0;
-    if (K == 1) {
-        int occ = 0, dev = 0, sms = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, kWThreads, smem) != cudaSuccess) return 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            return 0;
-        return occ * sms;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = K;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(K * 256, 1, 1);
-    cfg.blockDim = dim3(kWThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, f, &cfg) != cudaSuccess) return 0;
-    return clusters;
-}
+int configure_dfw(size_t smem, int K) { return cluster_slots((const void*)dfw_kernel(K), kWThreads, smem, K); }
 
 // grid: tile slots (clusters); each gets K blocks.
 cudaError_t launch_darkfield_wide(const DevPlan& P, int K, int grid, size_t smem, int n_tiles, const float* I,
@@ -770,29 +727,12 @@ cudaError_t launch_darkfield_wide(const DevPlan& P, int K, int grid, size_t smem
     if (!f || P.h != 16 * kWBN || P.w != P.h) return cudaErrorInvalidValue;
     const int slots = min(grid, n_tiles);
     if (slots < 1) return cudaErrorInvalidConfiguration;
-    if (K == 1) {
-        if (work) {
-            const cudaError_t e = cudaMemsetAsync(work, 0, sizeof(int), st);
-            if (e != cudaSuccess) return e;
-        }
-        f<<<slots, kWThreads, smem, st>>>(P, n_tiles, I, phi, spec, (char*)scratch, per_block, iters, tol, status,
-                                          counters, work);
-        return cudaGetLastError();
+    if (K == 1 && work) {
+        const cudaError_t e = cudaMemsetAsync(work, 0, sizeof(int), st);
+        if (e != cudaSuccess) return e;
     }
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = K;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(K * slots, 1, 1);
-    cfg.blockDim = dim3(kWThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, f, P, n_tiles, I, phi, spec, (char*)scratch, per_block, iters, tol, status,
-                              counters, (int*)nullptr);
+    return cluster_launch(f, K, slots, kWThreads, smem, st, P, n_tiles, I, phi, spec, (char*)scratch, per_block, iters,
+                          tol, status, counters, K == 1 ? work : (int*)nullptr);
 }
 
 }  // namespace apic
