@@ -14,7 +14,8 @@
 //   then x += alpha d, s -= alpha w, and d = s + beta d (folded into the next
 //   R1). Transforms, vectors and the partial sums of a thread and of a warp FP32;
 //   the sums across warps and the step lengths FP64 (the FP64 pipe is narrow, so it
-//   sees 16 values per reduction rather than every point).
+//   sees 16 values per reduction rather than every point, and one thread divides: a
+//   division by all 16 warps, twice an iteration, cost 2 % of the kernel).
 // Each image is solved in its own frame (x and y swapped when that makes the row
 // bands shorter) on its own grid: mx = 16 BX row points and my = 16 BY column
 // points, the cheapest supported pair on which both correlations are exact
@@ -39,6 +40,7 @@
 #include "../../include/apic.h"
 #include "internal.cuh"
 #include "regfft.cuh"
+#include "tmem.cuh"
 
 namespace apic {
 
@@ -65,18 +67,6 @@ constexpr int kTmemSlots = kDFThreads / 128;                  // warps per lane 
 constexpr int kTmemSlotCols = kTmemSlots > 0 ? (kTmemCols / kTmemSlots) & ~31 : 0;
 // every pass has at most 3 pair rounds (<= 96 pairs of columns over >= 32 half-warps)
 constexpr bool kTmemField = kDFThreads % 128 == 0 && kTmemSlotCols >= 96;
-
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float2 (&v)[16]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-                 :: "r"(taddr), "f"(v[0].x), "f"(v[0].y), "f"(v[1].x), "f"(v[1].y), "f"(v[2].x), "f"(v[2].y), "f"(v[3].x), "f"(v[3].y), "f"(v[4].x), "f"(v[4].y), "f"(v[5].x), "f"(v[5].y), "f"(v[6].x), "f"(v[6].y), "f"(v[7].x), "f"(v[7].y), "f"(v[8].x), "f"(v[8].y), "f"(v[9].x), "f"(v[9].y), "f"(v[10].x), "f"(v[10].y), "f"(v[11].x), "f"(v[11].y), "f"(v[12].x), "f"(v[12].y), "f"(v[13].x), "f"(v[13].y), "f"(v[14].x), "f"(v[14].y), "f"(v[15].x), "f"(v[15].y) : "memory");
-}
-// load and wait in one statement, so no use of v can be scheduled before the wait
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float2 (&v)[16]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
-                 "tcgen05.wait::ld.sync.aligned;"
-                 : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[2].x), "=f"(v[2].y), "=f"(v[3].x), "=f"(v[3].y), "=f"(v[4].x), "=f"(v[4].y), "=f"(v[5].x), "=f"(v[5].y), "=f"(v[6].x), "=f"(v[6].y), "=f"(v[7].x), "=f"(v[7].y), "=f"(v[8].x), "=f"(v[8].y), "=f"(v[9].x), "=f"(v[9].y), "=f"(v[10].x), "=f"(v[10].y), "=f"(v[11].x), "=f"(v[11].y), "=f"(v[12].x), "=f"(v[12].y), "=f"(v[13].x), "=f"(v[13].y), "=f"(v[14].x), "=f"(v[14].y), "=f"(v[15].x), "=f"(v[15].y) : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 struct HW {
     int t, hw;
@@ -747,10 +737,9 @@ __device__ __forceinline__ int df_solve(const DFCtx& c, const DevPlan& P, const 
         pass_rows_mask<BX>(w, twx, c.GQ, nQ, qmask);
         cols_times<BY, false>(c, twy, mx, c.GQ, mx, nQ, c.GU, LDU, nU);
         const float dw = pass_rows_out<BX>(w, twx, c.GU, LDU, nU, urp, P.dU_x + u_off, OutDot{c.wv, c.dv});
-        const double delta = block_sum2f(dw, c.red, par);
+        float af;
+        const double delta = block_sum2f_ratio<false>(dw, gamma, c.red, par, af);      // af = gamma / delta
         if (!(delta > 0)) break;
-        const double alpha = gamma / delta;
-        const float af = (float)alpha;
         float g2 = 0.f;
         for (int e = threadIdx.x; e < N; e += blockDim.x) {
             const float2 d = c.dv[e];
@@ -762,8 +751,7 @@ __device__ __forceinline__ int df_solve(const DFCtx& c, const DevPlan& P, const 
             c.sv[e] = sv;
             g2 += sv.x * sv.x + sv.y * sv.y;
         }
-        const double gnew = block_sum2f(g2, c.red, par);
-        bf = (float)(gnew / gamma);
+        const double gnew = block_sum2f_ratio<true>(g2, gamma, c.red, par, bf);        // bf = gnew / gamma
         gamma = gnew;
         conv = gnew <= stop;
     }
