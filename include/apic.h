@@ -216,7 +216,9 @@ apic_status apic_plan_set_df_grid(apic_plan* plan, int index, int mx, int my);
  * a second stream the plan owns, forked from and joined back to `stream`
  * (stream capture follows the fork), while the other tiles' earlier stages
  * run on the remaining SMs; a larger partial wave simply ends the darkfield
- * stage. Results are identical in every order.
+ * stage. Tiles beyond the last full wave that are not split off, and batches
+ * below one wave, are solved by clusters of several thread blocks per tile.
+ * Results are identical in every order and with any number of blocks.
  */
 apic_status apic_reconstruct_batch(apic_plan* plan, int n_tiles, const float* d_intensity,
                                    float* d_field, float* d_zernike, float* d_pupil,

@@ -97,8 +97,9 @@ struct apic_plan {
     int grid_dfr = 0;            // tile slots of the register darkfield kernel (blocks, or clusters of
                                  // df_cluster blocks for the wide kernel)
     int df_cluster = 1;          // blocks per tile of the wide darkfield kernel
-    int dfw_slots[3] = {0, 0, 0};   // wide kernel: tile slots with 1, 2, 4 blocks per tile
+    int df_slots[kMaxCluster + 1] = {};   // register darkfield kernels: tile slots with K blocks per tile
     int df_slots_alloc = 0;      // tile slots of each half of the darkfield scratch
+    bool df_rounds = true;       // small batches in rounds of several blocks per tile (off while autotuning)
     // host-buffer pipeline (apic_reconstruct_host), created on first use
     struct HostIO {
         bool ready = false;
@@ -210,6 +211,7 @@ apic_status upload(apic_plan* plan) {
     std::vector<int> ux, uy, up, ua, px, py, pp, pa, qx, qy, rp;
     std::vector<unsigned> qmask;
     int maxN = 1, maxM = 1, band_u = 1, band_p = 1, band_q = 1, max_mx = 16, max_mxy = 256;
+    int cl_mx = 16, cl_maxB = 1;
     const int mr = H.mr;
     for (const auto& d : H.df) {
         if (!d.used) continue;
@@ -290,6 +292,8 @@ apic_status upload(apic_plan* plan) {
         band_u = std::max(band_u, e.uy1 - e.uy0 + 1);
         band_p = std::max(band_p, e.py1 - e.py0 + 1);
         band_q = std::max(band_q, e.qy1 - e.qy0 + 1);
+        cl_mx = std::max(cl_mx, 16 * e.bx);
+        cl_maxB = std::max({cl_maxB, e.bx, e.by});
         e.qmask_off = (int)qmask.size();
         if (mr > 0) {   // Q membership per band row on the image's row grid, as 16-bit lane masks
             // x index xi = t + Bm k1 sits in lane(-slot) t, bit k1; 8 words per row, 16 on
@@ -316,6 +320,8 @@ apic_status upload(apic_plan* plan) {
     D.band_u = band_u;
     D.band_p = band_p;
     D.band_q = band_q;
+    D.cl_mx = cl_mx;
+    D.cl_maxB = cl_maxB;
     if (qmask.empty()) qmask.push_back(0u);
     const size_t o_df = A.add(dfs);
     const size_t o_ux = A.add(ux), o_uy = A.add(uy), o_up = A.add(up), o_ua = A.add(ua);
@@ -387,6 +393,16 @@ apic_status upload(apic_plan* plan) {
     return APIC_OK;
 }
 
+// Clusters of K blocks that the cluster kernel of tiles up to 256 pixels runs at once, for the
+// plan's current tables.
+void configure_clusters(apic_plan* plan) {
+    if (!plan->dfr_ok || plan->dev.mr == 512) return;
+    for (int K = 2; K <= kMaxCluster; ++K) {
+        plan->df_slots[K] = configure_dfc(plan->dev, K);
+        cudaGetLastError();
+    }
+}
+
 apic_status configure(apic_plan* plan) {
     const DevPlan& D = plan->dev;
     Launch& L = plan->L;
@@ -423,33 +439,28 @@ apic_status configure(apic_plan* plan) {
                                  : dfr_smem_bytes(D.mr / 16, D.h / 16, D.band_u, D.band_q, D.max_N);
         int dev_max = 0;
         cudaDeviceGetAttribute(&dev_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, plan->device);
-        if (smem <= (size_t)dev_max && wide) {
-            // blocks per tile: 1 by default (measured fastest: with 2 or 4 blocks per tile
-            // fewer tiles are in flight, but the cluster barriers and the passes' rows and
-            // columns split over more half-warps cost more than L2 residency gains); the
-            // autotuner times 1, 2 and 4
-            for (int i = 0; i < 3; ++i) {
-                plan->dfw_slots[i] = configure_dfw(smem, 1 << i);
-                cudaGetLastError();
-            }
-            const int pick = plan->dfw_slots[0] > 0 ? 0 : 1;
-            if (plan->dfw_slots[pick] > 0) {
+        if (smem <= (size_t)dev_max) {
+            // blocks per tile: 1 by default, the most tiles per second from a full wave on
+            // (launch_df takes more for smaller batches; for 512-pixel tiles the
+            // autotuner times 1, 2 and 4 and can settle on another default)
+            if (wide)
+                for (int K = 1; K <= kMaxCluster; ++K) {
+                    plan->df_slots[K] = configure_dfw(smem, K);
+                    cudaGetLastError();
+                }
+            else
+                plan->df_slots[1] = sms * configure_dfr(D.mr / 16, D.h / 16, smem);
+            const int pick = plan->df_slots[1] > 0 || !wide ? 1 : 2;
+            if (plan->df_slots[pick] > 0) {
                 plan->dfr_ok = true;
                 plan->smem_dfr = smem;
-                plan->df_cluster = 1 << pick;
-                plan->grid_dfr = plan->dfw_slots[pick];
+                plan->df_cluster = pick;
+                plan->grid_dfr = plan->df_slots[pick];
             }
-        } else if (smem <= (size_t)dev_max) {
-            const int occ = configure_dfr(D.mr / 16, D.h / 16, smem);
-            if (occ > 0) {
-                plan->dfr_ok = true;
-                plan->smem_dfr = smem;
-                plan->grid_dfr = sms * occ;
-            } else {
-                cudaGetLastError();
-            }
+            cudaGetLastError();
         }
     }
+    configure_clusters(plan);
     const bool legacy = (plan->params.flags & APIC_LEGACY_KERNELS) != 0;
     plan->use_kkr = plan->kkr_ok && !legacy;
     plan->use_reg = plan->dfr_ok && !legacy;
@@ -491,8 +502,8 @@ apic_status alloc_workspace(apic_plan* p) {
     // darkfield scratch for two waves of blocks: a batch's last partial wave runs
     // beside the full waves (reconstruct) on blocks of its own
     if (p->use_reg) {
-        // the wide kernel's scratch covers the most tile slots of any cluster size
-        p->df_slots_alloc = D.mr == 512 ? std::max({p->dfw_slots[0], p->dfw_slots[1], p->dfw_slots[2]}) : p->grid_dfr;
+        // the scratch covers the most tile slots of any cluster size
+        p->df_slots_alloc = D.mr == 512 ? *std::max_element(p->df_slots, p->df_slots + kMaxCluster + 1) : p->grid_dfr;
         p->df_per_block = D.mr == 512 ? dfw_scratch_bytes(D) : dfr_scratch_bytes(D);
         if ((s = dmalloc(p, &p->df_scratch, 2 * (size_t)p->df_slots_alloc * p->df_per_block)) != APIC_OK) return s;
     } else {
@@ -549,8 +560,110 @@ cudaError_t launch_df_on(apic_plan* p, int n_tiles, const float* I, const float*
                             status, p->d_counters, st);
 }
 
+// Ways to solve a round of tiles: K blocks per tile, at most `cap` tiles at once, in `t`
+// times the time of a round of one block per tile. Measured on a GB300, the darkfield
+// stage of as many tiles as run at once (a cluster's blocks share a GPC, so fewer than
+// SMs / K), in milliseconds:
+//   128 px, 8 + 16 images: 5.5 (151 tiles, K = 1), 4.2 (46, 3), 3.3 (28, 5), 3.2 (15, 8)
+//   256 px, 8 + 16: 15.6 (151, 1), 8.4 (46, 3), 6.7 (36, 4), 6.2 (23, 6), 5.0 (15, 8)
+//   512 px, 8 + 24: 69 (151, 1), 40 (76, 2), 29 (46, 3), 25.9 (36, 4), 21.6 (28, 5),
+//   20.3 (23, 6), 18.5 (15, 8), 15.1 (13, 10); K = 16 is no faster than 10 on one tile
+// 64-pixel tiles stay with one block (2.4 ms; clusters were slower).
+struct DfOption {
+    int K, cap;
+    double t;
+};
+
+std::vector<DfOption> df_options(const apic_plan* p) {
+    static const double t128[][2] = {{3, 0.77}, {5, 0.61}, {8, 0.59}};
+    static const double t256[][2] = {{3, 0.54}, {4, 0.43}, {6, 0.40}, {8, 0.32}};
+    static const double t512[][2] = {{2, 0.58}, {3, 0.42}, {4, 0.37}, {5, 0.31}, {6, 0.29}, {8, 0.27}, {10, 0.22}};
+    std::vector<DfOption> o{{1, p->grid_dfr, 1.0}};
+    auto add = [&](const double (*t)[2], int n) {
+        for (int i = 0; i < n; ++i) {
+            // clusters that run at once, and that the scratch of one wave holds
+            const int K = (int)t[i][0];
+            const size_t each = p->dev.mr == 512 ? p->df_per_block : dfc_scratch_bytes(p->dev);
+            const int cap = (int)std::min<size_t>(p->df_slots[K], p->df_slots_alloc * p->df_per_block / each);
+            if (cap > 0) o.push_back({K, cap, t[i][1]});
+        }
+    };
+    switch (p->dev.h) {
+        case 128: add(t128, 3); break;
+        case 256: add(t256, 4); break;
+        case 512: add(t512, 7); break;
+    }
+    return o;
+}
+
+// Rounds for n tiles (less than a full wave): the sequence of options with the least total
+// time, in round times of one block per tile (dynamic programming over the tiles left).
+double df_schedule(const apic_plan* p, int n, std::vector<DfOption>* rounds) {
+    const std::vector<DfOption> opt = df_options(p);
+    std::vector<double> best(n + 1, 0.0);
+    std::vector<int> pick(n + 1, 0);
+    for (int k = 1; k <= n; ++k) {
+        best[k] = 1e30;
+        for (int i = 0; i < (int)opt.size(); ++i) {
+            const double t = opt[i].t + best[std::max(0, k - opt[i].cap)];
+            if (t < best[k]) {
+                best[k] = t;
+                pick[k] = i;
+            }
+        }
+    }
+    if (rounds)
+        for (int k = n; k > 0; k -= opt[pick[k]].cap) rounds->push_back(opt[pick[k]]);
+    return best[n];
+}
+
+bool df_may_cluster(const apic_plan* p) { return p->use_reg && p->df_rounds && p->df_cluster == 1; }
+
+// Darkfield stage of a batch. One block per tile is the most tiles per second while it
+// keeps every SM busy; the tiles beyond the last full wave (all of a smaller batch) would
+// leave SMs idle for as long as a tile's chain of solves takes, so they go in rounds of
+// K blocks per tile (df_schedule). A tile's result is bit for bit the same with any K.
 cudaError_t launch_df(apic_plan* p, int n_tiles, const float* I, float2* spec, int32_t* status, cudaStream_t st) {
-    return launch_df_on(p, n_tiles, I, p->phi, spec, status, false, st);
+    if (!df_may_cluster(p)) return launch_df_on(p, n_tiles, I, p->phi, spec, status, false, st);
+    const DevPlan& D = p->dev;
+    const size_t in_tile = (size_t)D.n_img * D.h * D.w;
+    int a = n_tiles / df_wave(p) * df_wave(p);
+    if (a > 0) {
+        const cudaError_t e = launch_df_on(p, a, I, p->phi, spec, status, false, st);
+        if (e != cudaSuccess) return e;
+    }
+    std::vector<DfOption> rounds;
+    df_schedule(p, n_tiles - a, &rounds);
+    for (const DfOption& o : rounds) {
+        const int k = std::min(o.cap, n_tiles - a);
+        const float* Ia = I + (size_t)a * in_tile;
+        const float* ph = p->phi + (size_t)a * D.npup;
+        float2* sp = spec + (size_t)a * D.nap;
+        int32_t* stt = status ? status + a : nullptr;
+        cudaError_t e;
+        if (D.mr == 512)
+            e = launch_darkfield_wide(D, o.K, k, p->smem_dfr, k, Ia, ph, sp, p->df_scratch, p->df_per_block,
+                                      p->df_iters, p->df_tol, stt, p->d_counters, p->d_work, st);
+        else if (o.K == 1)
+            e = launch_df_on(p, k, Ia, ph, sp, stt, false, st, k);
+        else
+            e = launch_darkfield_cluster(D, o.K, k, k, Ia, ph, sp, p->df_scratch, p->df_iters, p->df_tol, stt,
+                                         p->d_counters, st);
+        if (e != cudaSuccess) return e;
+        if (a > 0) ++p->launches;
+        a += k;
+    }
+    return cudaSuccess;
+}
+
+// Whether r trailing tiles beyond m0 tiles of full waves are better solved after them, in
+// rounds of clusters (launch_df), than in the split order, where they take a whole round
+// but hide most of the other tiles' earlier stages: those take about kPre round times
+// per tile (2048 tiles of 512: 126 ms against rounds of 67 ms; 512 of 256: 5 ms
+// against 15.6 ms).
+bool df_rounds_beat_split(const apic_plan* p, int r, int m0) {
+    constexpr double kPre = 9e-4;
+    return df_may_cluster(p) && df_schedule(p, r, nullptr) + kPre * m0 < 1.0;
 }
 
 apic_status check_plan(const apic_plan* plan, int n_tiles) {
@@ -686,6 +799,10 @@ apic_status reconstruct(apic_plan* plan, apic_net* net, int mode, int n_tiles, c
         float* zt = zern + (size_t)t0 * APIC_N_ZERNIKE;
         int r = 0, m0 = nt, ma = nt, ml = nt;   // partial wave, full waves, their groups
         split_geometry(plan, nt, r, m0, ma, ml);
+        if (r > 0 && !hk && df_rounds_beat_split(plan, r, m0)) {
+            r = 0;
+            m0 = ma = ml = nt;
+        }
         // earlier stages of tiles [a, a + k) of the chunk; in the split order this runs
         // for the partial wave (a = m0) and then for the full waves (a = 0), so a stage's
         // interval starts with the first call and ends with the call for a = 0. cap > 0
@@ -1195,6 +1312,7 @@ apic_status apic_plan_set_df_grid(apic_plan* plan, int index, int mx, int my) {
         auto it = std::find(plan->allocs.begin(), plan->allocs.end(), old_tables);
         if (it != plan->allocs.end()) plan->allocs.erase(it);
     }
+    configure_clusters(plan);
     return APIC_OK;
 }
 
@@ -1603,11 +1721,12 @@ apic_status apic_plan_autotune(apic_plan* plan, int n_tiles, const float* I, dou
     // stitched spectrum, so repeated runs see the same system
     const bool had_reg = plan->use_reg;
     const bool wide = D.mr == 512;
+    plan->df_rounds = false;             // the variants themselves, not a small batch's rounds
     const int had_k = plan->df_cluster, had_grid = plan->grid_dfr;
     void* scratch[2] = {nullptr, nullptr};
     size_t per_block[2] = {wide ? dfw_scratch_bytes(D) : dfr_scratch_bytes(D), df_scratch_bytes(D)};
     const int slots_alloc[2] = {
-        wide ? std::max({plan->dfw_slots[0], plan->dfw_slots[1], plan->dfw_slots[2]}) : plan->grid_dfr,
+        wide ? *std::max_element(plan->df_slots, plan->df_slots + kMaxCluster + 1) : plan->grid_dfr,
         plan->L.grid_df};
     scratch[had_reg ? 0 : 1] = plan->df_scratch;
     int best_k = had_k, best_grid = had_grid;
@@ -1623,9 +1742,9 @@ apic_status apic_plan_autotune(apic_plan* plan, int n_tiles, const float* I, dou
         plan->df_slots_alloc = slots_alloc[v];
         if (v == 0 && wide) {      // the wide kernel at each cluster size: blocks per tile 1, 2, 4
             for (int i = 0; i < 3 && err == cudaSuccess; ++i) {
-                if (plan->dfw_slots[i] <= 0) continue;
+                if (plan->df_slots[1 << i] <= 0) continue;
                 plan->df_cluster = 1 << i;
-                plan->grid_dfr = plan->dfw_slots[i];
+                plan->grid_dfr = plan->df_slots[1 << i];
                 err = timed([&] { return launch_df(plan, n_tiles, I, plan->spec, stt, st); }, ms[4 + i]);
                 if (err == cudaSuccess && (ms[2] < 0 || ms[4 + i] < ms[2])) {
                     ms[2] = ms[4 + i];
@@ -1659,6 +1778,7 @@ apic_status apic_plan_autotune(apic_plan* plan, int n_tiles, const float* I, dou
         plan->df_cluster = had_k;
         plan->grid_dfr = had_grid;
     }
+    plan->df_rounds = true;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaStreamDestroy(st);

@@ -1,0 +1,99 @@
+"""Small batches: the darkfield solves of a tile spread over a cluster of blocks.
+
+A batch below a full wave is solved in rounds of several blocks per tile, the number
+chosen by the batch size. Covered here: every choice at each tile size, rounds of
+different kinds within one batch and graph replay.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+from paper_2407_20469_gb300 import apic, learn, synth  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+def _run(plan, I, n):
+    H = plan.info.out_h
+    f = torch.full((n, H, 2 * H), 7.0, dtype=torch.float32, device="cuda")
+    z = torch.empty((n, 15), dtype=torch.float32, device="cuda")
+    st = torch.full((n,), -1, dtype=torch.int32, device="cuda")
+    plan.reconstruct_batch(n, I[:n].contiguous(), f, z, None, st)
+    torch.cuda.synchronize()
+    return f, z, st
+
+
+def _tiles(tile, ill, n, up=2):
+    plan = apic.Plan.from_illumination(tile, ill, max_tiles=n, upsample=up)
+    uv, zern, blank = learn.draw_tiles(n, 3, learn.field_table())
+    if up == 2:
+        return plan, learn.simulate(plan, zern, blank, 3)
+    p2 = apic.Plan.from_illumination(tile, ill, max_tiles=1)
+    return plan, learn.simulate(p2, zern, blank, 3)
+
+
+@pytest.mark.parametrize("tile,ill,up,sizes", [
+    (64, "8+16", 2, (1, 40, 100)),
+    (128, "8+16", 2, (1, 7, 20, 37, 60, 100)),
+    (256, "8+16", 2, (1, 9, 20, 33, 45, 60, 100)),
+    (256, "12+22", 3, (2, 30)),
+    (512, "8+24", 2, (1, 9, 24, 30, 50)),
+])
+def test_batch_size_does_not_change_a_tile(tile, ill, up, sizes):
+    """The tiles of a small batch (clusters of every size in use, rounds of different sizes)
+    are bit for bit those of a full wave (one block per tile)."""
+    il = {"8+16": synth.illumination, "8+24": synth.illumination_8_24, "12+22": synth.illumination_12_22}[ill]()
+    W = apic.Plan.from_illumination(tile, il, max_tiles=1).info.df_wave
+    plan, I = _tiles(tile, il, W, up)
+    f_ref, z_ref, s_ref = _run(plan, I, W)
+    assert int(s_ref.max()) == 0
+    for n in sizes:
+        f, z, st = _run(plan, I, n)
+        assert torch.equal(z, z_ref[:n]) and torch.equal(st, s_ref[:n]), n
+        assert torch.equal(f, f_ref[:n]), n
+
+
+@pytest.mark.parametrize("mx,my", [(192, 192), (192, 144), (192, 128), (192, 96), (160, 128), (160, 96), (144, 144)])
+def test_every_solve_grid_in_a_cluster(mx, my):
+    """Each (row, column) grid of the 256-pixel solve, forced on every image it is exact for:
+    one tile (a cluster) against the same tile in a full wave."""
+    ill = synth.illumination()
+    W = apic.Plan.from_illumination(256, ill, max_tiles=1).info.df_wave
+    plan, I = _tiles(256, ill, W)
+    for i in range(plan.info.n_df):
+        try:
+            plan.set_df_grid(i, mx, my)
+        except apic.ApicError:
+            pass
+    assert any(plan.df_grid(i)[1:] == (mx, my) for i in range(plan.info.n_df))
+    f_ref, _, _ = _run(plan, I, W)
+    f, _, _ = _run(plan, I, 1)
+    assert torch.equal(f[0], f_ref[0])
+
+
+def test_skipped_tiles_in_a_cluster_round():
+    """Background tiles leave their cluster at once; the others are what they are alone."""
+    ill = synth.illumination()
+    T = 11
+    zern = learn.coefficients(learn.field_table(), np.zeros((T, 2), np.float32))
+    blank = np.zeros(T, dtype=bool)
+    blank[::3] = True
+    plan = apic.Plan.from_illumination(256, ill, max_tiles=T, bg_contrast=0.02, flags=apic.APIC_SKIP_BACKGROUND)
+    I = learn.simulate(plan, zern, blank, 5)
+    f, z, st = _run(plan, I, T)
+    keep = torch.as_tensor(np.nonzero(~blank)[0], device="cuda")
+    f1, z1, _ = _run(plan, I[keep], len(keep))
+    assert torch.count_nonzero(f[torch.as_tensor(np.nonzero(blank)[0], device="cuda")]) == 0
+    assert torch.equal(f[keep], f1) and torch.equal(z[keep], z1)
+
+
+def test_cluster_round_replays_from_a_graph():
+    ill = synth.illumination()
+    plan, I = _tiles(128, ill, 3)
+    f0, z0, _ = _run(plan, I, 3)
+    f, z = torch.zeros_like(f0), torch.zeros_like(z0)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        plan.reconstruct_batch(3, I, f, z)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(f, f0) and torch.equal(z, z0)
