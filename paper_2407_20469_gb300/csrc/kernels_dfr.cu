@@ -29,7 +29,9 @@
 // gu_ld(B): column passes are conflict free per warp - m + 2 where they move column
 // pairs as 16-byte accesses, m + 1 where single columns); GQ, the column-major known
 // field p of the longer grids and b on Q live in the block's global scratch
-// (L2-resident; data read once - the images - is loaded evict-first). The setup
+// (L2-resident; data read once - the images - is loaded evict-first). GQ is stored in
+// 4 x 4 tiles (t4grid.cuh): the column passes touch 4 lines per instruction instead of 16
+// (512 tiles of 256: 64.2 -> 59.7 ms). The setup
 // transforms of each image reuse the shared-memory space of GU. One block per tile
 // (persistent); images of a tile are sequential. Each pass is a separate
 // (non-inlined) function so registers are allocated per pass.
@@ -40,6 +42,7 @@
 #include "../../include/apic.h"
 #include "internal.cuh"
 #include "regfft.cuh"
+#include "t4grid.cuh"
 #include "tmem.cuh"
 
 namespace apic {
@@ -188,8 +191,9 @@ struct MidTimesFieldT {
 
 // ---- passes
 
-// rows of a band: scatter val(e) at x = px[e], inverse transform along x, store rows of G (row stride ld)
-template <int B, class Val>
+// rows of a band: scatter val(e) at x = px[e], inverse transform along x, store rows of G
+// (row stride ld; T4: tiled, ld columns)
+template <int B, bool T4, class Val>
 __device__ __noinline__ void pass_rows_in(HW w, const float2* tw, float2* G, int ld, int nrows, const int* rp,
                                           const int* px, Val val) {
     constexpr int m = 16 * B;
@@ -206,9 +210,16 @@ __device__ __noinline__ void pass_rows_in(HW w, const float2* tw, float2* G, int
         __syncwarp(w.mask);
         fft_alpha<B, true>(v, o, h, tw);
         if (w.t < B) {
-            float2* row = G + (size_t)b * ld;
+            if constexpr (T4) {
+                const T4Lane L(w.t);
+                float2* row = G + t4_row(b, ld);
 #pragma unroll
-            for (int k1 = 0; k1 < 16; ++k1) row[w.t + B * k1] = o[k1];
+                for (int k1 = 0; k1 < 16; ++k1) row[L.at(B * k1)] = o[k1];
+            } else {
+                float2* row = G + (size_t)b * ld;
+#pragma unroll
+                for (int k1 = 0; k1 < 16; ++k1) row[w.t + B * k1] = o[k1];
+            }
         }
     }
 }
@@ -237,6 +248,14 @@ __device__ __noinline__ float pass_rows_out(HW w, const float2* tw, const float2
     return acc;
 }
 
+// Offset of row t, column x of a grid with ld columns (T4: tiled) - row t + 16 j is 16 j ld
+// further in both layouts. Pairs of columns x, x + 1 (x even) are adjacent, in 16-byte
+// aligned places where ld is even.
+template <bool T4>
+__device__ __forceinline__ int grid_at(int t, int x, int ld) {
+    return T4 ? t4_row(t, ld) + t4_col(x) : t * ld + x;
+}
+
 // columns x < ncols of a grid whose columns have 16 B points: the ni band rows of Gi
 // (row stride ldi) are the input at column indices 0..ni - 1, the rest zero; inverse
 // along y, mid, forward along y; column indices 0..no - 1 stored as the band rows of
@@ -247,7 +266,7 @@ __device__ __noinline__ float pass_rows_out(HW w, const float2* tw, const float2
 // and writes its own columns, so Gi and Go may be the same grid; the known-field
 // values of the column are loaded after the first transform. Ends with
 // __syncthreads.
-template <int B, class Mid>
+template <int B, bool T4I, bool T4O, class Mid>
 __device__ __noinline__ void pass_cols(HW w, const float2* tw, int ncols, const float2* Gi, int ldi, int ni,
                                        float2* Go, int ldo, int no, Mid mid) {
     static_assert(!Mid::kTmem, "TMEM operations need the paired pass");
@@ -258,7 +277,7 @@ __device__ __noinline__ void pass_cols(HW w, const float2* tw, int ncols, const 
 #pragma unroll
         for (int j = 0; j < B; ++j) {
             const int bb = w.t + 16 * j;
-            v[j] = bb < ni ? Gi[(size_t)bb * ldi + x] : make_float2(0.f, 0.f);
+            v[j] = bb < ni ? Gi[grid_at<T4I>(w.t, x, ldi) + 16 * j * ldi] : make_float2(0.f, 0.f);
         }
         fft_alpha<B, true>(v, o, h, tw);
         // the known field of the column, loaded once the inputs are consumed (loading it
@@ -275,7 +294,7 @@ __device__ __noinline__ void pass_cols(HW w, const float2* tw, int ncols, const 
 #pragma unroll
             for (int k1 = 0; k1 < B; ++k1) {
                 const int bb = w.t + 16 * k1;
-                if (bb < no) Go[(size_t)bb * ldo + x] = v[k1];
+                if (bb < no) Go[grid_at<T4O>(w.t, x, ldo) + 16 * k1 * ldo] = v[k1];
             }
         }
     }
@@ -286,7 +305,7 @@ __device__ __noinline__ void pass_cols(HW w, const float2* tw, int ncols, const 
 // x, x + 1 together (fft_alpha2 / fft_beta2), so every lane works in the DFT_16 step
 // and each pass makes half as many round trips per half-warp. ncols is even; a grid
 // with an even row stride (16-byte aligned rows) moves each pair as one 16-byte access.
-template <int B, class Mid>
+template <int B, bool T4I, bool T4O, class Mid>
 __device__ __noinline__ void pass_cols2(HW w, const float2* tw, int ncols, const float2* Gi, int ldi, int ni,
                                         float2* Go, int ldo, int no, Mid mid) {
     constexpr int m = 16 * B;
@@ -303,7 +322,7 @@ __device__ __noinline__ void pass_cols2(HW w, const float2* tw, int ncols, const
         for (int j = 0; j < B; ++j) {
             const int bb = w.t + 16 * j;
             if (bb < ni) {
-                const float2* g = Gi + (size_t)bb * ldi + x;
+                const float2* g = Gi + grid_at<T4I>(w.t, x, ldi) + 16 * j * ldi;
                 if (vin) {
                     const float4 q = *reinterpret_cast<const float4*>(g);
                     va[j] = make_float2(q.x, q.y);
@@ -335,7 +354,7 @@ __device__ __noinline__ void pass_cols2(HW w, const float2* tw, int ncols, const
             for (int k1 = 0; k1 < B; ++k1) {
                 const int bb = w.t + 16 * k1;
                 if (bb < no) {
-                    float2* g = Go + (size_t)bb * ldo + x;
+                    float2* g = Go + grid_at<T4O>(w.t, x, ldo) + 16 * k1 * ldo;
                     if (vout) {
                         *reinterpret_cast<float4*>(g) = make_float4(va[k1].x, va[k1].y, vb[k1].x, vb[k1].y);
                     } else {
@@ -352,7 +371,7 @@ __device__ __noinline__ void pass_cols2(HW w, const float2* tw, int ncols, const
 // pass_cols for columns too long to pair in the lanes (B > 8): each half-warp takes the
 // column pair x, x + 1 and transforms the two in turn, so that the pair still moves as
 // one 16-byte access per row on grids with an even row stride. ncols is even.
-template <int B, class Mid>
+template <int B, bool T4I, bool T4O, class Mid>
 __device__ __noinline__ void pass_cols_seq2(HW w, const float2* tw, int ncols, const float2* Gi, int ldi, int ni,
                                             float2* Go, int ldo, int no, Mid mid) {
     static_assert(!Mid::kTmem, "TMEM operations need the paired pass");
@@ -365,7 +384,7 @@ __device__ __noinline__ void pass_cols_seq2(HW w, const float2* tw, int ncols, c
         for (int j = 0; j < B; ++j) {
             const int bb = w.t + 16 * j;
             if (bb < ni) {
-                const float2* g = Gi + (size_t)bb * ldi + x;
+                const float2* g = Gi + grid_at<T4I>(w.t, x, ldi) + 16 * j * ldi;
                 if (vin) {
                     const float4 q = *reinterpret_cast<const float4*>(g);
                     va[j] = make_float2(q.x, q.y);
@@ -399,7 +418,7 @@ __device__ __noinline__ void pass_cols_seq2(HW w, const float2* tw, int ncols, c
             for (int k1 = 0; k1 < B; ++k1) {
                 const int bb = w.t + 16 * k1;
                 if (bb < no) {
-                    float2* g = Go + (size_t)bb * ldo + x;
+                    float2* g = Go + grid_at<T4O>(w.t, x, ldo) + 16 * k1 * ldo;
                     if (vout) {
                         *reinterpret_cast<float4*>(g) = make_float4(va[k1].x, va[k1].y, vb[k1].x, vb[k1].y);
                     } else {
@@ -414,16 +433,19 @@ __device__ __noinline__ void pass_cols_seq2(HW w, const float2* tw, int ncols, c
 }
 
 // column pass on a 16 B grid: paired columns where two fit a half-warp, column pairs
-// in turn up to B = 12, single columns beyond
-template <int B, class Mid>
+// in turn up to B = 12, single columns beyond. (160 columns are two and a half rounds of
+// pairs for 32 half-warps; giving the last half round out as single columns, one to a
+// half-warp, was 5 % slower over the whole kernel: it adds a function to the hot loop's code
+// and 8-byte accesses in the place of 16-byte ones.)
+template <int B, bool T4I, bool T4O, class Mid>
 __device__ __forceinline__ void cols(HW w, const float2* tw, int ncols, const float2* Gi, int ldi, int ni,
                                      float2* Go, int ldo, int no, Mid mid) {
     if constexpr (2 * B <= 16)
-        pass_cols2<B>(w, tw, ncols, Gi, ldi, ni, Go, ldo, no, mid);
+        pass_cols2<B, T4I, T4O>(w, tw, ncols, Gi, ldi, ni, Go, ldo, no, mid);
     else if constexpr (B <= 12)
-        pass_cols_seq2<B>(w, tw, ncols, Gi, ldi, ni, Go, ldo, no, mid);
+        pass_cols_seq2<B, T4I, T4O>(w, tw, ncols, Gi, ldi, ni, Go, ldo, no, mid);
     else
-        pass_cols<B>(w, tw, ncols, Gi, ldi, ni, Go, ldo, no, mid);
+        pass_cols<B, T4I, T4O>(w, tw, ncols, Gi, ldi, ni, Go, ldo, no, mid);
 }
 
 // rows of Q in place: forward along x, keep the Q lags, inverse along x. Ends with __syncthreads.
@@ -432,12 +454,12 @@ __device__ __noinline__ void pass_rows_mask(HW w, const float2* tw, float2* G, i
     constexpr int m = 16 * B;
     const HalfWarp h = w.h();
     for (int b = w.hw; b < nrows; b += kHW) {
-        float2* row = G + (size_t)b * m;
+        float2* row = G + t4_row(b, m) + t4_col(w.t);           // columns t + 16 j: 64 j further
         // lane t's Q membership of x = t + B k1 (bit k1)
         const unsigned bits = qmask[(size_t)b * 8 + (w.t >> 1)] >> (16 * (w.t & 1));
         float2 v[B], o[16];
 #pragma unroll
-        for (int j = 0; j < B; ++j) v[j] = row[w.t + 16 * j];
+        for (int j = 0; j < B; ++j) v[j] = row[64 * j];
         fft_alpha<B, false>(v, o, h, tw);
         if (w.t < B) {
 #pragma unroll
@@ -446,7 +468,7 @@ __device__ __noinline__ void pass_rows_mask(HW w, const float2* tw, float2* G, i
         }
         fft_beta<B, true>(o, v, h, tw);
 #pragma unroll
-        for (int k1 = 0; k1 < B; ++k1) row[w.t + 16 * k1] = v[k1];
+        for (int k1 = 0; k1 < B; ++k1) row[64 * k1] = v[k1];
     }
     __syncthreads();
 }
@@ -534,10 +556,10 @@ __device__ __noinline__ void pass_rows_rhs(HW w, const float2* tw, float2* GQ, i
     const HalfWarp h = w.h();
     const float inv_m2 = 1.f / (float)(m * m);
     for (int b = w.hw; b < nQ; b += kHW) {
-        float2* row = GQ + (size_t)b * m;
+        float2* row = GQ + t4_row(b, m);
         float2 v[B], o[16];
 #pragma unroll
-        for (int j = 0; j < B; ++j) v[j] = row[w.t + 16 * j];
+        for (int j = 0; j < B; ++j) v[j] = row[t4_col(w.t) + 64 * j];
         fft_alpha<B, false>(v, o, h, tw);
         if (w.t < B) {
 #pragma unroll
@@ -558,8 +580,9 @@ __device__ __noinline__ void pass_rows_rhs(HW w, const float2* tw, float2* GQ, i
         __syncwarp(w.mask);
         fft_alpha<B, true>(v, o, h, tw);
         if (w.t < B) {
+            const T4Lane L(w.t);
 #pragma unroll
-            for (int k1 = 0; k1 < 16; ++k1) row[w.t + B * k1] = o[k1];
+            for (int k1 = 0; k1 < 16; ++k1) row[L.at(B * k1)] = o[k1];
         }
     }
     __syncthreads();
@@ -622,7 +645,7 @@ size_t dfr_smem_bytes(int B, int BN, int band_u, int band_q, int max_N) {
 // rows, b on Q.
 size_t dfr_scratch_bytes(const DevPlan& P) {
     const int m = P.mr, n = P.h;
-    size_t s = (size_t)(P.band_q > P.band_p ? P.band_q : P.band_p) * m * sizeof(float2);  // GQ
+    size_t s = (size_t)t4_rows(std::max(P.band_q, P.band_p)) * m * sizeof(float2);  // GQ (tiled)
     s += std::max((size_t)m * m, (size_t)P.band_q * n) * sizeof(float2);           // PF / F(I) rows
     s += (size_t)P.max_M * sizeof(float2);                                         // b on Q
     return (s + 255) & ~(size_t)255;
@@ -646,13 +669,13 @@ __host__ __device__ constexpr bool uses_tmem(int B) { return kTmemField && (B ==
 
 // Column pass that multiplies by the scaled field p s or its conjugate: from TMEM on
 // paired grids, else from the column-major copy in global scratch
-template <int BY, bool CONJ>
+template <int BY, bool CONJ, bool T4I, bool T4O>
 __device__ __forceinline__ void cols_times(const DFCtx& c, const float2* tw, int m, const float2* Gi, int ldi, int ni,
                                            float2* Go, int ldo, int no) {
     if constexpr (2 * BY <= 16 && kTmemField)
-        cols<BY>(c.w, tw, m, Gi, ldi, ni, Go, ldo, no, MidTimesFieldT<CONJ>{c.tm});
+        cols<BY, T4I, T4O>(c.w, tw, m, Gi, ldi, ni, Go, ldo, no, MidTimesFieldT<CONJ>{c.tm});
     else
-        cols<BY>(c.w, tw, m, Gi, ldi, ni, Go, ldo, no, MidTimesField<BY, CONJ>{c.PF});
+        cols<BY, T4I, T4O>(c.w, tw, m, Gi, ldi, ni, Go, ldo, no, MidTimesField<BY, CONJ>{c.PF});
 }
 
 // plain twiddle table of a 16 G-point grid of a solve on the 16 B-point register grid
@@ -690,7 +713,7 @@ __device__ __forceinline__ int df_solve(const DFCtx& c, const DevPlan& P, const 
     // band rows of the known field P (Eq. 11) along x on the row grid, staged in GQ
     // (row stride mx), then p s on the column grid (s = 1 / (mx my): the two
     // unnormalised transforms around each product)
-    pass_rows_in<BX>(w, twx, c.GQ, mx, nP, prp, P.dP_x + p_off, pval);
+    pass_rows_in<BX, true>(w, twx, c.GQ, mx, nP, prp, P.dP_x + p_off, pval);
     __syncthreads();
     // (the columns passes transform each band as if it started at row 0, so the field
     // carries the ramp W^((uy0 - qy0) y) of the U <-> Q passes and W^(-py0 y) for its
@@ -698,29 +721,29 @@ __device__ __forceinline__ int df_solve(const DFCtx& c, const DevPlan& P, const 
     const float scale = 1.f / ((float)mx * (float)my);
     const int shift = (((uy0 - qy0 - py0) % my) + my) % my;
     if constexpr (2 * BY <= 16 && kTmemField) {
-        cols<BY>(w, twy, mx, c.GQ, mx, nP, c.GQ, mx, 0,
+        cols<BY, true, true>(w, twy, mx, c.GQ, mx, nP, c.GQ, mx, 0,
                  MidStoreFieldT{c.tm, scale, grid_table(P, BY, B), shift, BY});
         tmem_wait_st();
     } else {
-        cols<BY>(w, twy, mx, c.GQ, mx, nP, c.GQ, mx, 0,
+        cols<BY, true, true>(w, twy, mx, c.GQ, mx, nP, c.GQ, mx, 0,
                  MidStoreField<BY>{c.PF, scale, grid_table(P, BY, B), shift});
     }
     // |p|^2 (blind to the P band's start) times W^(qy0 y): its transform's Q band from row 0
     const MidAbs2<B> abs2{nullptr, P.tw_r, ((qy0 % m) + m) % m};
     // b -= P * P on Q (16 B grid), then the rows of b inverse along x on the row grid
     if constexpr (BX == B) {
-        cols<B>(w, c.tw_m, m, c.GQ, m, nP, c.GQ, m, nQ, abs2);
+        cols<B, true, true>(w, c.tw_m, m, c.GQ, m, nP, c.GQ, m, nQ, abs2);
         pass_rows_rhs<B, true>(w, c.tw_m, c.GQ, nQ, qrp, P.dQ_x + q_off, c.bq);
     } else {
-        pass_rows_in<B>(w, c.tw_m, c.GQ, m, nP, prp, P.dP_x + p_off, pval);
+        pass_rows_in<B, true>(w, c.tw_m, c.GQ, m, nP, prp, P.dP_x + p_off, pval);
         __syncthreads();
-        cols<B>(w, c.tw_m, m, c.GQ, m, nP, c.GQ, m, nQ, abs2);
+        cols<B, true, true>(w, c.tw_m, m, c.GQ, m, nP, c.GQ, m, nQ, abs2);
         pass_rows_rhs<B, false>(w, c.tw_m, c.GQ, nQ, qrp, P.dQ_x + q_off, c.bq);
-        pass_rows_in<BX>(w, twx, c.GQ, mx, nQ, qrp, P.dQ_x + q_off, ValB{c.bq});
+        pass_rows_in<BX, true>(w, twx, c.GQ, mx, nQ, qrp, P.dQ_x + q_off, ValB{c.bq});
         __syncthreads();
     }
     // s = d = C^H b
-    cols_times<BY, false>(c, twy, mx, c.GQ, mx, nQ, c.GU, LDU, nU);
+    cols_times<BY, false, true, false>(c, twy, mx, c.GQ, mx, nQ, c.GU, LDU, nU);
     const float g0 = pass_rows_out<BX>(w, twx, c.GU, LDU, nU, urp, P.dU_x + u_off, OutStart{c.sv, c.dv, c.xv});
     int par = 0;
     const double gamma0 = block_sum2f(g0, c.red, par);
@@ -731,11 +754,11 @@ __device__ __forceinline__ int df_solve(const DFCtx& c, const DevPlan& P, const 
     int it = 0;
     float bf = 0.f;                  // first direction: d = s
     for (; it < iters && !conv; ++it) {
-        pass_rows_in<BX>(w, twx, c.GU, LDU, nU, urp, P.dU_x + u_off, ValNextDir{c.sv, c.dv, bf});
+        pass_rows_in<BX, false>(w, twx, c.GU, LDU, nU, urp, P.dU_x + u_off, ValNextDir{c.sv, c.dv, bf});
         __syncthreads();
-        cols_times<BY, true>(c, twy, mx, c.GU, LDU, nU, c.GQ, mx, nQ);
+        cols_times<BY, true, false, true>(c, twy, mx, c.GU, LDU, nU, c.GQ, mx, nQ);
         pass_rows_mask<BX>(w, twx, c.GQ, nQ, qmask);
-        cols_times<BY, false>(c, twy, mx, c.GQ, mx, nQ, c.GU, LDU, nU);
+        cols_times<BY, false, true, false>(c, twy, mx, c.GQ, mx, nQ, c.GU, LDU, nU);
         const float dw = pass_rows_out<BX>(w, twx, c.GU, LDU, nU, urp, P.dU_x + u_off, OutDot{c.wv, c.dv});
         float af;
         const double delta = block_sum2f_ratio<false>(dw, gamma, c.red, par, af);      // af = gamma / delta
@@ -826,7 +849,7 @@ k_darkfield_reg(DevPlan P, int n_tiles, const float* __restrict__ I, const float
     c.xv = reinterpret_cast<float2*>(sbase + SL.x);
     char* base = scratch + (size_t)blockIdx.x * per_block;
     c.GQ = reinterpret_cast<float2*>(base);
-    c.PF = c.GQ + (size_t)(P.band_q > P.band_p ? P.band_q : P.band_p) * m;   // column-major p, or F(I) rows
+    c.PF = c.GQ + (size_t)t4_rows(max(P.band_q, P.band_p)) * m;   // column-major p, or F(I) rows
     c.bq = c.PF + (size_t)max(m * m, P.band_q * n);
 
     // tiles taken one at a time from the launch's counter (a block that meets skipped
