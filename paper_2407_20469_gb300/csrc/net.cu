@@ -98,25 +98,18 @@ __global__ void __launch_bounds__(512, 1) k_features(DevPlan P, int n_tiles, con
     for (int prob = blockIdx.x; prob < nprob; prob += gridDim.x) {
         const int tile = prob / kIn, i = prob - tile * kIn;
         const float* img = I + ((size_t)tile * P.n_img + i) * n * n;
-        // the image's sum: per thread as a float pair (rowsum.cuh; an FP64 add per pixel kept
-        // the FP64 pipe busy for a quarter of the kernel's time), across threads in FP64
+        // the image's sum on the way: per thread as a float pair (rowsum.cuh; an FP64 add per
+        // pixel kept the FP64 pipe busy for a quarter of the kernel's time), across threads in
+        // FP64
         FF sum = {0.f, 0.f};
-        const float4* img4 = reinterpret_cast<const float4*>(img);
-        for (int q = threadIdx.x; q < n * n / 4; q += blockDim.x) {
-            const float4 v = img4[q];
-            const float x[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const FF t = ff_two_sum(sum.hi, x[e]);
-                sum = {t.hi, sum.lo + t.lo};
-            }
-        }
-        const double s = block_sum((double)sum.hi + (double)sum.lo, red);
-        const float inv_dc = s > 0 ? (float)(1.0 / s) : 0.f;
         for (int r = hw; r < n; r += NHW) {
             float2 v[BN], o[S][16];
 #pragma unroll
-            for (int j = 0; j < BN; ++j) v[j] = make_float2(img[(size_t)r * n + t + 16 * j], 0.f);
+            for (int j = 0; j < BN; ++j) {
+                v[j] = make_float2(img[(size_t)r * n + t + 16 * j], 0.f);
+                const FF q = ff_two_sum(sum.hi, v[j].x);
+                sum = {q.hi, sum.lo + q.lo};
+            }
             fft_a<BN, false>(v, o, h, tw);
 #pragma unroll
             for (int sl = 0; sl < S; ++sl)
@@ -129,7 +122,8 @@ __global__ void __launch_bounds__(512, 1) k_features(DevPlan P, int n_tiles, con
                     }
                 }
         }
-        __syncthreads();
+        const double s = block_sum((double)sum.hi + (double)sum.lo, red);     // (a barrier)
+        const float inv_dc = s > 0 ? (float)(1.0 / s) : 0.f;
         float* f = feat + (size_t)tile * kCrop * kCrop * kIn + i;
         for (int c = hw; c < kCrop; c += NHW) {
             float2 v[BN], o[S][16];
