@@ -1,9 +1,42 @@
-// cluster.cuh - set-up and launch of kernels that run on clusters of K blocks (K = 1: plain blocks).
+// cluster.cuh - kernels whose unit of work is taken by one block or by a cluster of K
+// blocks: device helpers, set-up and launch (K = 1: plain blocks).
 #pragma once
 
 #include "common.cuh"
 
 namespace apic {
+
+__device__ __forceinline__ uint32_t cta_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cta_count() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+
+// Barrier of all threads of the unit's blocks (release / acquire at cluster scope); a
+// block barrier without a cluster.
+template <bool CL>
+__device__ __forceinline__ void tile_sync() {
+    if constexpr (!CL) {
+        __syncthreads();
+    } else {
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+}
+
+// Load of global data that another block of the cluster may have written: from L2.
+template <bool CL, class T>
+__device__ __forceinline__ T ldx(const T* p) {
+    if constexpr (CL)
+        return __ldcg(p);
+    else
+        return *p;
+}
 
 inline void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, int K, int slots, int threads,
                            size_t smem, cudaStream_t st) {

@@ -19,8 +19,8 @@
 //    cluster barriers, one behind each pass.
 // What bounds it: the chain of five passes per iteration, each a half-warp's one or two
 // transforms deep (about 1.6 k cycles each), and the barriers (about 1 k each). Measured
-// (GB300, darkfield stage of one tile, 8 + 16 images): 128 pixels 5.0 -> 3.0 ms, 256 pixels
-// 14.6 -> 4.8 ms with 8 blocks. With the grids in L2 instead (the one-block kernel's passes
+// (GB300, darkfield stage of one tile, 8 + 16 images): 128 pixels 5.0 -> 2.7 ms, 256 pixels
+// 14.6 -> 4.3 ms with 8 blocks. With the grids in L2 instead (the one-block kernel's passes
 // split over a cluster) the same tiles took 4.9 and 8.3 ms: the release of every barrier
 // waits for the stores to reach L2, and each pass then loads from there. More than 8
 // blocks gain nothing: a share is then less than a half-warp's transform each.
@@ -31,6 +31,7 @@
 #include <algorithm>
 
 #include "../../include/apic.h"
+#include "cluster.cuh"
 #include "internal.cuh"
 #include "regfft.cuh"
 #include "t4grid.cuh"
@@ -41,15 +42,18 @@ namespace apic {
 constexpr int kClThreads = 320;                 // 20 half-warps: the 18-20 columns, 16-17 Q rows of a share of 1/8 (256 px)
 constexpr int kClHW = kClThreads / 16;
 constexpr int kClTmemCols = 512;
+constexpr int kClQWords = 8;                    // Q membership words per band row (two 16-bit masks each)
 constexpr int kClTmemSlot = 160;                // TMEM columns per thread: 10 warps, three per lane quarter
 
 // Shared memory of one block (byte offsets, 16-aligned). The half-warp areas of the
 // camera-grid setup transforms alias the CG's areas, vectors and slabs up to cq; the cq
 // slab is apart (it receives the known field's rows, then b's, while the setup runs).
-// cu: U rows' columns on their way into C1, then (ru) the U rows out of C2; the two are
-// never live together.
+// cu: U rows' columns on their way into C1, then the U rows out of C2; the two are never
+// live together. urp, ux, qm: the image's U row pointers, the points' positions on the row
+// grid, and the Q masks of the block's rows - the acquire of a cluster barrier drops the
+// L1 cache, so tables in global memory cost each pass an L2 round trip or two.
 struct ClSmem {
-    size_t vec, cu, rq, cq, tw, tab, red, total;
+    size_t vec, cu, rq, cq, tw, tab, urp, ux, qm, red, total;
 };
 
 __host__ __device__ inline size_t cl_align(size_t b) { return (b + 15) & ~(size_t)15; }
@@ -70,7 +74,10 @@ __host__ __device__ inline ClSmem cl_smem_layout(int BN, int B, int K, int maxB,
     L.cq = cl_max(cg_end, setup);
     L.tw = L.cq + cl_align((size_t)(band_q > band_p ? band_q : band_p) * lc * c);
     L.tab = L.tw + cl_align((size_t)2 * 16 * (BN + B + 2 * maxB) * c);
-    L.red = L.tab + cl_align((size_t)(mx + band_q + band_u) * sizeof(uint32_t));
+    L.urp = L.tab + cl_align((size_t)(mx + band_q + band_u) * sizeof(uint32_t));
+    L.ux = L.urp + cl_align((size_t)(band_u + 1) * sizeof(int));
+    L.qm = L.ux + cl_align((size_t)max_N * sizeof(uint16_t));
+    L.red = L.qm + cl_align((size_t)cl_share(band_q, K) * kClQWords * sizeof(unsigned));
     L.total = L.red + 64 * sizeof(double);
     return L;
 }
@@ -94,16 +101,6 @@ namespace {
 
 __device__ __forceinline__ int sfreqc(int i, int n) { return i < n / 2 ? i : i - n; }
 
-__device__ __forceinline__ uint32_t cl_ctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t cl_nctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
 // the cluster-wide address of a shared-memory address of this block in block `rank`
 __device__ __forceinline__ uint32_t cl_map(uint32_t a, uint32_t rank) {
     uint32_t r;
@@ -113,10 +110,7 @@ __device__ __forceinline__ uint32_t cl_map(uint32_t a, uint32_t rank) {
 __device__ __forceinline__ void cl_st(uint32_t a, float2 v) {
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
 }
-__device__ __forceinline__ void cl_sync() {
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
+__device__ __forceinline__ void cl_sync() { tile_sync<true>(); }
 
 // Half-warp hw of the block, lane t; hs its transform area; tm the thread's TMEM columns.
 struct ClLane {
@@ -147,11 +141,6 @@ struct ClValKnown {      // P(c) = O_known(K) exp(j phi(c)); the spectrum is wri
         return cmul(__ldcg(sp + ap[e]), make_float2(cs, sn));
     }
 };
-struct ClValDir {        // d
-    const float2* dv;
-    __device__ float2 operator()(int e) const { return dv[e]; }
-};
-
 // ---- per-column operations on o[s][k1], the value at y = (t + 16 s) + B k1
 template <int B>
 struct ClMidStore {      // p s W^(shift y) into the thread's TMEM columns (wt: W_16B^j)
@@ -215,7 +204,32 @@ __device__ __noinline__ void cl_rows_in(ClLane w, const float2* tw, int r0, int 
     }
 }
 
-// the known field's rows on the camera grid, into the tiled grid GP in global scratch
+// the block's U rows of the direction d: as cl_rows_in with the tables in shared memory
+template <int B>
+__device__ __noinline__ void cl_rows_dir(ClLane w, const float2* tw, int r0, int nr, const int* urp, const uint16_t* ux,
+                                         const float2* dv, ClDst dst) {
+    const HalfWarp h = w.h();
+    for (int b = r0 + w.hw; b < r0 + nr; b += kClHW) {
+#pragma unroll
+        for (int j = 0; j < B; ++j) w.hs[w.t + 16 * j] = make_float2(0.f, 0.f);
+        __syncwarp(w.mask);
+        const int e1 = urp[b + 1];
+        for (int e = urp[b] + w.t; e < e1; e += 16) w.hs[ux[e]] = dv[e];
+        __syncwarp(w.mask);
+        float2 v[B], o[1][16];
+#pragma unroll
+        for (int j = 0; j < B; ++j) v[j] = w.hs[w.t + 16 * j];
+        __syncwarp(w.mask);
+        fft_a<B, true>(v, o, h, tw);
+        const uint32_t at = dst.off + b * dst.step;
+        if (w.t < B) {
+#pragma unroll
+            for (int k1 = 0; k1 < 16; ++k1) cl_st(dst.tab[w.t + B * k1] + at, o[0][k1]);
+        }
+    }
+}
+
+// the known field's rows on the register grid, into the tiled grid GP in global scratch
 // (every block reads its columns from L2)
 template <int B>
 __device__ __noinline__ void cl_rows_known(ClLane w, const float2* tw, int r0, int nr, const int* rp, const int* px,
@@ -275,11 +289,11 @@ __device__ __noinline__ void cl_cols(ClLane w, const float2* tw, int rounds, int
     }
 }
 
-// the block's Q rows: forward along x, keep the Q lags (qmask: `words` words per band row
-// of two 16-bit masks, bit k1 of mask t + 16 s for x index (t + 16 s) + B k1), inverse along x.
+// the block's Q rows: forward along x, keep the Q lags (qmask: per row of the block, words of
+// two 16-bit masks, bit k1 of mask t for x index t + B k1), inverse along x.
 template <int B>
 __device__ __noinline__ void cl_rows_mask(ClLane w, const float2* tw, int r0, int nr, const float2* G, int ld,
-                                          const unsigned* qmask, int words, ClDst dst) {
+                                          const unsigned* qmask, ClDst dst) {
     constexpr int S = Slots<B>::value;
     const HalfWarp h = w.h();
     for (int i = w.hw; i < nr; i += kClHW) {
@@ -288,7 +302,7 @@ __device__ __noinline__ void cl_rows_mask(ClLane w, const float2* tw, int r0, in
 #pragma unroll
         for (int s = 0; s < S; ++s) {
             const int ls = w.t + 16 * s;
-            qw[s] = ls < B ? qmask[(size_t)b * words + (ls >> 1)] >> (16 * (ls & 1)) : 0u;
+            qw[s] = ls < B ? qmask[i * kClQWords + (ls >> 1)] >> (16 * (ls & 1)) : 0u;
         }
         float2 v[B], o[S][16];
 #pragma unroll
@@ -310,16 +324,14 @@ __device__ __noinline__ void cl_rows_mask(ClLane w, const float2* tw, int r0, in
 // every block (wT: w's address in block t's shared memory, lanes t < K)
 template <int B>
 __device__ __noinline__ void cl_rows_out(ClLane w, const float2* tw, int r0, int nr, const float2* G, int ld,
-                                         const int* rp, const int* px, uint32_t wa, int K) {
-    constexpr int m = 16 * B, S = Slots<B>::value;
+                                         const int* urp, const uint16_t* ux, uint32_t wa, int K) {
+    constexpr int S = Slots<B>::value;
     const HalfWarp h = w.h();
     for (int i = w.hw; i < nr; i += kClHW) {
         const int b = r0 + i;
         float2 v[B], o[S][16];
 #pragma unroll
         for (int j = 0; j < B; ++j) v[j] = G[(w.t + 16 * j) * ld + i];
-        const int e0 = rp[b] + w.t, e1 = rp[b + 1];
-        int xn = e0 < e1 ? px[e0] : 0;
         fft_a<B, false>(v, o, h, tw);
 #pragma unroll
         for (int s = 0; s < S; ++s)
@@ -328,10 +340,9 @@ __device__ __noinline__ void cl_rows_out(ClLane w, const float2* tw, int r0, int
                 for (int k1 = 0; k1 < 16; ++k1) w.hs[w.t + 16 * s + B * k1] = o[s][k1];
             }
         __syncwarp(w.mask);
-        for (int e = e0; e < e1; e += 16) {
-            const int xc = xn;
-            if (e + 16 < e1) xn = px[e + 16];
-            const float2 val = w.hs[freq_index(xc, m)];
+        const int e1 = urp[b + 1];
+        for (int e = urp[b] + w.t; e < e1; e += 16) {
+            const float2 val = w.hs[ux[e]];
             for (int r = 0; r < K; ++r) cl_st(cl_map(wa + 8 * e, r), val);
         }
         __syncwarp(w.mask);
@@ -481,8 +492,8 @@ __device__ __forceinline__ double cl_sum_ratio(Part part, double num, double* re
     }
     __syncthreads();
     if (warp == 0) {
-        double t = lane < kRefWarps ? r[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        double t = r[lane & (kRefWarps - 1)];
+        for (int o = kRefWarps / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
         if (lane == 0) {
             r[31] = t;
             r[30] = OVER ? t / num : num / t;
@@ -531,7 +542,7 @@ __device__ __forceinline__ int cl_solve(const ClCtx& c, const DevPlan& P, const 
     const int u_off = D.u_off, p_off = D.p_off, q_off = D.q_off;
     const int uy0 = D.uy0, qy0 = D.qy0, py0 = D.py0;
     const int N = D.N, nU = D.uy1 - uy0 + 1, nQ = D.qy1 - qy0 + 1, nP = D.py1 - py0 + 1;
-    const int *urp = P.d_rowptr + D.urp, *qrp = P.d_rowptr + D.qrp, *prp = P.d_rowptr + D.prp;
+    const int *qrp = P.d_rowptr + D.qrp, *prp = P.d_rowptr + D.prp;
     // shares: columns, U rows, Q rows, P rows, camera-grid and register-grid columns
     const int sc = cl_share(mx, K), su = cl_share(nU, K), sq = cl_share(nQ, K), spn = cl_share(nP, K);
     const int sn = cl_share(n, K), sm = cl_share(m, K);
@@ -545,6 +556,12 @@ __device__ __forceinline__ int cl_solve(const ClCtx& c, const DevPlan& P, const 
     for (int i = threadIdx.x; i < mx; i += kClThreads) tabC[i] = cl_map(c.base, i / sc) + 8 * (i % sc);
     for (int i = threadIdx.x; i < nQ; i += kClThreads) tabQ[i] = cl_map(c.base, i / sq) + 8 * (i % sq);
     for (int i = threadIdx.x; i < nU; i += kClThreads) tabU[i] = cl_map(c.base, i / su) + 8 * (i % su);
+    int* urp = reinterpret_cast<int*>(c.smem + c.L.urp);
+    uint16_t* ux = reinterpret_cast<uint16_t*>(c.smem + c.L.ux);
+    unsigned* qm = reinterpret_cast<unsigned*>(c.smem + c.L.qm);
+    for (int i = threadIdx.x; i <= nU; i += kClThreads) urp[i] = P.d_rowptr[D.urp + i];
+    for (int i = threadIdx.x; i < N; i += kClThreads) ux[i] = (uint16_t)freq_index(P.dU_x[u_off + i], mx);
+    for (int i = threadIdx.x; i < nq * kClQWords; i += kClThreads) qm[i] = P.d_qmask[D.qmask_off + q0 * kClQWords + i];
     const float2 *wx = cl_table(P, BX, B), *wy = cl_table(P, BY, B);
     make_step_twiddles(c.tw_x, wx, BX);
     make_step_twiddles(c.tw_y, wy, BY);
@@ -585,7 +602,7 @@ __device__ __forceinline__ int cl_solve(const ClCtx& c, const DevPlan& P, const 
     cl_sync();
     cl_cols<BY>(c.w, c.tw_y, rounds, c0, nc, CQ, lc, nQ, nU, ClMidTimes<BY, false>{}, toRU);
     cl_sync();
-    cl_rows_out<BX>(c.w, c.tw_x, u0, nu, CU, lu, urp, P.dU_x + u_off, wa, K);
+    cl_rows_out<BX>(c.w, c.tw_x, u0, nu, CU, lu, urp, ux, wa, K);
     cl_sync();
     for (int e = threadIdx.x; e < N; e += kClThreads) {
         const float2 v = wv[e];
@@ -612,15 +629,15 @@ __device__ __forceinline__ int cl_solve(const ClCtx& c, const DevPlan& P, const 
     for (; it < iters && !conv; ++it) {
         for (int e = threadIdx.x; e < N; e += kClThreads) dv[e] = cadd(sv[e], cscale(dv[e], bf));
         __syncthreads();
-        cl_rows_in<BX>(c.w, c.tw_x, u0, nu, urp, P.dU_x + u_off, ClValDir{dv}, toCU);
+        cl_rows_dir<BX>(c.w, c.tw_x, u0, nu, urp, ux, dv, toCU);
         cl_sync();
         cl_cols<BY>(c.w, c.tw_y, rounds, c0, nc, CU, lc, nU, nQ, ClMidTimes<BY, true>{}, toRQ);
         cl_sync();
-        cl_rows_mask<BX>(c.w, c.tw_x, q0, nq, RQ, lq, P.d_qmask + D.qmask_off, P.qmask_words, toCQ);
+        cl_rows_mask<BX>(c.w, c.tw_x, q0, nq, RQ, lq, qm, toCQ);
         cl_sync();
         cl_cols<BY>(c.w, c.tw_y, rounds, c0, nc, CQ, lc, nQ, nU, ClMidTimes<BY, false>{}, toRU);
         cl_sync();
-        cl_rows_out<BX>(c.w, c.tw_x, u0, nu, CU, lu, urp, P.dU_x + u_off, wa, K);
+        cl_rows_out<BX>(c.w, c.tw_x, u0, nu, CU, lu, urp, ux, wa, K);
         cl_sync();
         float af;
         const double delta = cl_sum_ratio<false>(
@@ -698,8 +715,8 @@ k_darkfield_cluster(DevPlan P, ClSmem L, int n_tiles, const float* __restrict__ 
     c.smem = reinterpret_cast<char*>(smem4);
     c.base = (uint32_t)__cvta_generic_to_shared(c.smem);
     c.L = L;
-    c.K = (int)cl_nctarank();
-    c.rank = (int)cl_ctarank();
+    c.K = (int)cta_count();
+    c.rank = (int)cta_rank();
     const int slot = blockIdx.x / c.K, nslots = gridDim.x / c.K;
     c.tw_n = reinterpret_cast<float2*>(c.smem + L.tw);
     c.tw_m = c.tw_n + 2 * 16 * BN;

@@ -1,6 +1,5 @@
 // kernels_dfc.cu - the cluster darkfield kernel (dfc.cuh): tiles of 128 pixels, set-up
 // and launch.
-#include "cluster.cuh"
 #include "dfc.cuh"
 
 namespace apic {

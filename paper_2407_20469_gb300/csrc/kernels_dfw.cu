@@ -67,38 +67,6 @@ struct HWw {
     __device__ HalfWarp h() const { return HalfWarp{t, mask, hs}; }
 };
 
-__device__ __forceinline__ unsigned cta_rank() {
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-__device__ __forceinline__ unsigned cta_count() {
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-
-// Barrier of all threads of the K blocks of a tile (release / acquire at cluster
-// scope); a block barrier when K = 1.
-template <bool CL>
-__device__ __forceinline__ void tile_sync() {
-    if constexpr (!CL) {
-        __syncthreads();
-    } else {
-        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-    }
-}
-
-// Load of scratch data that another block of the cluster may have written: from L2.
-template <bool CL>
-__device__ __forceinline__ float2 ldx(const float2* p) {
-    if constexpr (!CL)
-        return *p;
-    else
-        return __ldcg(p);
-}
-
 // The sum of a U row's values over the half-warp, into entry b of the list rs of every
 // block of the tile (its own through distributed shared memory as well).
 template <bool CL>
