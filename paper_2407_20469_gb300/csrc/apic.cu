@@ -99,6 +99,7 @@ struct apic_plan {
     int df_cluster = 1;          // blocks per tile of the wide darkfield kernel
     int df_slots[kMaxCluster + 1] = {};   // register darkfield kernels: tile slots with K blocks per tile
     int df_slots_alloc = 0;      // tile slots of each half of the darkfield scratch
+    int kk_slots[kMaxCluster + 1] = {};   // Kramers-Kronig problems at once with K (a power of 2) blocks each
     bool df_rounds = true;       // small batches in rounds of several blocks per tile (off while autotuning)
     // host-buffer pipeline (apic_reconstruct_host), created on first use
     struct HostIO {
@@ -424,13 +425,14 @@ apic_status configure(apic_plan* plan) {
     plan->kkr_ok = plan->dfr_ok = false;
     if (D.h == D.w && (D.h == 64 || D.h == 128 || D.h == 256 || D.h == 512)) {
         const size_t smem = kkr_smem_bytes(D.h / 16);
-        const int occ = configure_kkr(D.h / 16, smem);
-        if (occ > 0) {
+        for (int K = 1; K <= kMaxCluster; K *= 2) {
+            plan->kk_slots[K] = configure_kkr(D.h / 16, smem, K);
+            cudaGetLastError();
+        }
+        if (plan->kk_slots[1] > 0) {
             plan->kkr_ok = true;
             plan->smem_kkr = smem;
-            plan->grid_kkr = sms * occ;
-        } else {
-            cudaGetLastError();
+            plan->grid_kkr = plan->kk_slots[1];
         }
     }
     if (D.mr > 0) {
@@ -524,14 +526,37 @@ apic_status alloc_workspace(apic_plan* p) {
     return APIC_OK;
 }
 
-// Kramers-Kronig stage on `blocks` blocks (<= 0: the plan's grid) with the given scratch.
+// Kramers-Kronig stage on at most `blocks` blocks (<= 0: the plan's grid) and `grids` n x n
+// grids of the given scratch (<= 0: the plan's). K blocks per problem (tile and image): the K
+// with the least rounds x time of a round, measured on a GB300 (milliseconds per round; the
+// results do not depend on K):
+//   512 px: 0.39 with one block, 0.22 with 2, 0.13 with 4, 0.074 with 8 (16: no faster)
+//   256 px: 0.107, 0.068, 0.044, 0.034;   128 px: 0.046, 0.036, 0.027, 0.027
+// Two blocks at 512 pixels also keep half as many grids in flight (152 MB): 96 tiles
+// 2.50 -> 2.43 ms, 25 tiles 0.83 -> 0.67.
 cudaError_t launch_kk_any(apic_plan* p, int blocks, int n_tiles, const float* I, float2* xdisc, float2* scratch,
-                          const int32_t* status, cudaStream_t st) {
-    if (p->use_kkr)
-        return launch_kk_reg(p->dev, blocks > 0 ? std::min(blocks, p->grid_kkr) : p->grid_kkr, p->smem_kkr, n_tiles,
-                             I, xdisc, scratch, status, st);
-    return launch_kk_grid(p->dev, blocks > 0 ? std::min(blocks, p->L.grid_kk) : p->L.grid_kk, p->L.smem_kk, n_tiles,
-                          I, xdisc, scratch, status, st);
+                          const int32_t* status, cudaStream_t st, int grids = 0) {
+    if (p->use_kkr) {
+        static const double t[4][4] = {{1, 9, 9, 9}, {1, 0.78, 0.60, 0.60}, {1, 0.64, 0.42, 0.33}, {1, 0.57, 0.34, 0.20}};
+        const double* tk = t[p->dev.h == 512 ? 3 : p->dev.h == 256 ? 2 : p->dev.h == 128 ? 1 : 0];
+        const int most = blocks > 0 ? std::min(blocks, p->grid_kkr) : p->grid_kkr, nprob = n_tiles * p->dev.n_bf;
+        int K = 1, slots = 0;
+        double best = 1e30;
+        for (int i = 0; i < 4; ++i) {
+            int s = std::min(p->kk_slots[1 << i], most >> i);
+            if (grids > 0) s = std::min(s, grids);
+            const double v = s > 0 ? (nprob + s - 1) / s * tk[i] : 1e30;
+            if (v < best) {
+                best = v;
+                K = 1 << i;
+                slots = s;
+            }
+        }
+        return launch_kk_reg(p->dev, K, slots, p->smem_kkr, n_tiles, I, xdisc, scratch, status, st);
+    }
+    const int grid = blocks > 0 ? std::min(blocks, p->L.grid_kk) : p->L.grid_kk;
+    return launch_kk_grid(p->dev, grids > 0 ? std::min(grid, grids) : grid, p->L.smem_kk, n_tiles, I, xdisc, scratch,
+                          status, st);
 }
 
 // Darkfield blocks of one full wave (the grid of the selected kernel).
@@ -1353,8 +1378,8 @@ apic_status apic_kk_spectra_noalloc(apic_plan* plan, int n_tiles, const float* I
     if (n_tiles == 0) return APIC_OK;
     float2* scratch = nullptr;
     APIC_TRY_CUDA(noalloc_scratch(dev, &scratch));
-    const int blocks = (int)std::min<size_t>(cap / per_block, (size_t)std::max(plan->L.grid_kk, plan->grid_kkr));
-    APIC_TRY_LAUNCH(launch_kk_any(plan, blocks, n_tiles, I, (float2*)xdisc, scratch, nullptr, (cudaStream_t)stream));
+    const int grids = (int)std::min<size_t>(cap / per_block, (size_t)std::max(plan->L.grid_kk, plan->grid_kkr));
+    APIC_TRY_LAUNCH(launch_kk_any(plan, 0, n_tiles, I, (float2*)xdisc, scratch, nullptr, (cudaStream_t)stream, grids));
     return APIC_OK;
 }
 

@@ -112,8 +112,8 @@ cudaError_t launch_kk(const DevPlan& P, const Launch& L, int n_tiles, const floa
 cudaError_t launch_kk_grid(const DevPlan& P, int grid, size_t smem, int n_tiles, const float* I, float2* xdisc,
                            float2* scratch, const int32_t* status, cudaStream_t st);
 size_t kkr_smem_bytes(int BN);
-int configure_kkr(int BN, size_t smem);
-cudaError_t launch_kk_reg(const DevPlan& P, int grid, size_t smem, int n_tiles, const float* I, float2* xdisc,
+int configure_kkr(int BN, size_t smem, int K);   // K blocks per problem: problems that run at once
+cudaError_t launch_kk_reg(const DevPlan& P, int K, int slots, size_t smem, int n_tiles, const float* I, float2* xdisc,
                           float2* scratch, const int32_t* status, cudaStream_t st);
 // Measured FMA throughput (flop/s) of the current device's CUDA cores, FP32 or FP64 (kernels_peak.cu).
 cudaError_t measure_fma_rate(int precision, double* flops_per_s);
@@ -175,7 +175,7 @@ cudaError_t launch_darkfield_wide(const DevPlan& P, int K, int grid, size_t smem
                                   cudaStream_t st);
 
 // Network features (net.cu): feat [n_tiles][64][64][8] from the first 8 images
-// of each stack; `scratch` holds h * 64 complex values per block of `grid`.
+// of each stack, on at most `grid` SMs; `scratch` holds h * h complex values for each.
 cudaError_t launch_features(const DevPlan& P, int grid, int n_tiles, const float* I, float* feat, float2* scratch,
                             cudaStream_t st);
 size_t feature_floats();

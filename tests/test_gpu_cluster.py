@@ -97,3 +97,22 @@ def test_cluster_round_replays_from_a_graph():
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(f, f0) and torch.equal(z, z0)
+
+
+@pytest.mark.parametrize("tile,sizes", [(64, (1, 30)), (128, (1, 3, 30)), (256, (1, 2, 4, 9, 30)), (512, (1, 4, 9, 20))])
+def test_kramers_kronig_does_not_depend_on_the_blocks_per_problem(tile, sizes):
+    """Batches of every size class (8 to 1 blocks per problem) and the allocation-free entry
+    point (few grids, many blocks each) give the same spectra bit for bit."""
+    ill = synth.illumination()
+    n = max(sizes)
+    plan, I = _tiles(tile, ill, n)
+    shape = (plan.info.n_bf, plan.info.n_pupil, 2)
+    ref = torch.empty((n,) + shape, device="cuda")
+    plan.kk_spectra(n, I, ref)
+    for k in sizes:
+        x = torch.zeros((k,) + shape, device="cuda")
+        plan.kk_spectra(k, I[:k].contiguous(), x)
+        assert torch.equal(x, ref[:k]), k
+        x.zero_()
+        plan.kk_spectra_noalloc(k, I[:k].contiguous(), x)
+        assert torch.equal(x, ref[:k]), k
