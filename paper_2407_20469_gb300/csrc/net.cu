@@ -81,10 +81,18 @@ struct Layout {
 // keep the 64 columns kx in [-32, 32), forward transform of those columns,
 // keep ky in [-32, 32), log of the magnitude relative to the DC term (the
 // image sum). Output NHWC: feat[tile][ky + 32][kx + 32][image].
+// Three blocks of 256 threads per SM up to 256 pixels (as many as the scratch of n x n values
+// per SM holds), one of 512 at 512: at 256 pixels the kernel waits for its shared-memory
+// exchanges and loads, and 24 warps hide more of that than 16 do.
 template <int BN>
-__global__ void __launch_bounds__(512, 1) k_features(DevPlan P, int n_tiles, const float* __restrict__ I,
-                                                     float* __restrict__ feat, float2* __restrict__ scratch) {
-    constexpr int n = 16 * BN, HWS = HWSize<BN>::value, NHW = 32, S = Slots<BN>::value;
+struct FeatCfg {
+    static constexpr int threads = BN <= 16 ? 256 : 512, blocks = BN == 16 ? 3 : BN == 8 ? 2 : 1;
+};
+
+template <int BN>
+__global__ void __launch_bounds__(FeatCfg<BN>::threads, FeatCfg<BN>::blocks)
+k_features(DevPlan P, int n_tiles, const float* __restrict__ I, float* __restrict__ feat, float2* __restrict__ scratch) {
+    constexpr int n = 16 * BN, HWS = HWSize<BN>::value, NHW = FeatCfg<BN>::threads / 16, S = Slots<BN>::value;
     extern __shared__ float4 smem4[];
     float2* hw_area = reinterpret_cast<float2*>(smem4);
     float2* tw = hw_area + NHW * HWS;
@@ -148,7 +156,7 @@ __global__ void __launch_bounds__(512, 1) k_features(DevPlan P, int n_tiles, con
 }
 
 size_t features_smem(int BN) {
-    return (size_t)32 * std::max(17 * BN, 16 * (BN + 1)) * sizeof(float2) + (size_t)2 * 16 * BN * sizeof(float2);
+    return (size_t)(BN <= 16 ? 16 : 32) * std::max(17 * BN, 16 * (BN + 1)) * sizeof(float2) + (size_t)2 * 16 * BN * sizeof(float2);
 }
 
 // ------------------------------------------------------------------ GEMM
@@ -412,37 +420,29 @@ int blocks_for(size_t n) { return (int)std::max<size_t>(1, std::min<size_t>((n +
 
 }  // namespace net
 
-// Features of n_tiles tiles (the first 8 images of each stack) with the plan's
-// register transforms; `scratch` holds h * 64 complex values per block.
+// Features of n_tiles tiles (the first 8 images of each stack) with the plan's register
+// transforms on at most `grid` SMs; `scratch` holds h * h complex values for each of them
+// (a block uses h * 64).
 cudaError_t launch_features(const DevPlan& P, int grid, int n_tiles, const float* I, float* feat, float2* scratch,
                             cudaStream_t st) {
     using namespace net;
     const int BN = P.h / 16;
     const size_t smem = features_smem(BN);
-    grid = std::min(grid, n_tiles * kIn);
-    if (grid < 1) return cudaSuccess;
-    cudaError_t e = cudaSuccess;
+    auto launch = [&](auto kernel, int threads, int per_sm) -> cudaError_t {
+        const int blocks = std::min(grid * per_sm, n_tiles * kIn);
+        if (blocks < 1) return cudaSuccess;
+        const cudaError_t e = raise_smem_limit((const void*)kernel, smem);
+        if (e != cudaSuccess) return e;
+        kernel<<<blocks, threads, smem, st>>>(P, n_tiles, I, feat, scratch);
+        return cudaGetLastError();
+    };
     switch (BN) {
-        case 4:
-            e = raise_smem_limit((const void*)k_features<4>, smem);
-            if (e == cudaSuccess) k_features<4><<<grid, 512, smem, st>>>(P, n_tiles, I, feat, scratch);
-            break;
-        case 8:
-            e = raise_smem_limit((const void*)k_features<8>, smem);
-            if (e == cudaSuccess) k_features<8><<<grid, 512, smem, st>>>(P, n_tiles, I, feat, scratch);
-            break;
-        case 16:
-            e = raise_smem_limit((const void*)k_features<16>, smem);
-            if (e == cudaSuccess) k_features<16><<<grid, 512, smem, st>>>(P, n_tiles, I, feat, scratch);
-            break;
-        case 32:
-            e = raise_smem_limit((const void*)k_features<32>, smem);
-            if (e == cudaSuccess) k_features<32><<<grid, 512, smem, st>>>(P, n_tiles, I, feat, scratch);
-            break;
+        case 4: return launch(k_features<4>, FeatCfg<4>::threads, FeatCfg<4>::blocks);
+        case 8: return launch(k_features<8>, FeatCfg<8>::threads, FeatCfg<8>::blocks);
+        case 16: return launch(k_features<16>, FeatCfg<16>::threads, FeatCfg<16>::blocks);
+        case 32: return launch(k_features<32>, FeatCfg<32>::threads, FeatCfg<32>::blocks);
         default: return cudaErrorInvalidValue;
     }
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
 }
 
 size_t feature_floats() { return (size_t)net::kCrop * net::kCrop * net::kIn; }
