@@ -238,6 +238,24 @@ __device__ void chol_solve12(const double* L, const double* b, double* x) {
     }
 }
 
+// The 12 basis differences of row r: three 16-byte loads (scalar loads of a 48-byte row by
+// 32 lanes take 12 instructions of 12 lines each)
+struct Row12 {
+    float a[12];
+    __device__ Row12(const float* __restrict__ rows, int r) {
+        const float4* p = reinterpret_cast<const float4*>(rows) + (size_t)3 * r;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float4 v = __ldg(p + q);
+            a[4 * q] = v.x;
+            a[4 * q + 1] = v.y;
+            a[4 * q + 2] = v.z;
+            a[4 * q + 3] = v.w;
+        }
+    }
+    __device__ float operator[](int z) const { return a[z]; }
+};
+
 // Refinement passes c <- c + LS(wrap(beta - D c)) from the coefficients in
 // cc / cf (shared); returns the sum of squared wrapped residuals of the rows
 // at the final coefficients (every thread gets it).
@@ -246,8 +264,9 @@ __device__ double value_passes(const DevPlan& P, const float* beta, int passes, 
     float g[12];
     for (int pass = 0; pass < passes; ++pass) {
         for (int z = 0; z < 12; ++z) g[z] = 0.f;
+#pragma unroll 2
         for (int r = threadIdx.x; r < P.nrows; r += blockDim.x) {
-            const float* A = P.row_A + (size_t)r * 12;
+            const Row12 A(P.row_A, r);
             float pred = 0.f;
             for (int z = 0; z < 12; ++z) pred += A[z] * cf[z];
             const float e = wrap_pi(beta[r] - pred);
@@ -264,8 +283,9 @@ __device__ double value_passes(const DevPlan& P, const float* beta, int passes, 
         __syncthreads();
     }
     double res = 0;
+#pragma unroll 2
     for (int r = threadIdx.x; r < P.nrows; r += blockDim.x) {
-        const float* A = P.row_A + (size_t)r * 12;
+        const Row12 A(P.row_A, r);
         float pred = 0.f;
         for (int z = 0; z < 12; ++z) pred += A[z] * cf[z];
         const float e = wrap_pi(beta[r] - pred);
@@ -309,12 +329,12 @@ __global__ void __launch_bounds__(kThreads) k_aberration(DevPlan P, int n_tiles,
         float g[12];
         for (int z = 0; z < 12; ++z) g[z] = 0.f;
         for (int r = threadIdx.x; r < P.nrows; r += blockDim.x) {
-            const float* A = P.row_A + (size_t)r * 12;
+            const Row12 A(P.row_A, r);
             const float br = beta[r];
             const int nb[2] = {P.row_nx[r], P.row_ny[r]};
             for (int d = 0; d < 2; ++d) {
                 if (nb[d] < 0) continue;
-                const float* A2 = P.row_A + (size_t)nb[d] * 12;
+                const Row12 A2(P.row_A, nb[d]);
                 const float e = wrap_pi(beta[nb[d]] - br);
                 for (int z = 0; z < 12; ++z) g[z] += (A2[z] - A[z]) * e;
             }
