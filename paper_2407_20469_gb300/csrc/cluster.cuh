@@ -38,6 +38,17 @@ __device__ __forceinline__ T ldx(const T* p) {
         return *p;
 }
 
+// Stores a value at this address of shared memory in the cluster's first block.
+template <class T>
+__device__ __forceinline__ void st_first(T* p, T v) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)));
+    if constexpr (sizeof(T) == 8)
+        asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(a), "l"(*reinterpret_cast<long long*>(&v)) : "memory");
+    else
+        asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(a), "r"(*reinterpret_cast<int*>(&v)) : "memory");
+}
+
 inline void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, int K, int slots, int threads,
                            size_t smem, cudaStream_t st) {
     attr.id = cudaLaunchAttributeClusterDimension;

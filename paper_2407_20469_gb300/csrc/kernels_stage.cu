@@ -5,6 +5,7 @@
 #include <math.h>
 
 #include "../../include/apic.h"
+#include "cluster.cuh"
 #include "passes.cuh"
 #include "zernike.h"
 
@@ -15,21 +16,27 @@ namespace apic {
 // tiles below the threshold and stacks with negative or non-finite values.
 // Each thread sums its own pixels in FP32 (a few hundred values), the block
 // combines the partial sums in FP64; the darkfield images are only checked.
-__global__ void __launch_bounds__(kThreads) k_background(DevPlan P, int n_tiles, const float* __restrict__ I,
+// The tile's images are dealt to the K blocks of a cluster; the first block adds the
+// images' values in image order, so the result does not depend on K.
+constexpr int kMaxBF = 255;                 // plans take no more NA-matching images
+
+__global__ void __launch_bounds__(kThreads) k_background(DevPlan P, const float* __restrict__ I,
                                                          float* __restrict__ c2, int32_t* __restrict__ status,
                                                          float thresh2, int learned) {
     __shared__ double red[64];
-    const int tile = blockIdx.x;
-    if (tile >= n_tiles) return;
+    __shared__ double value[kMaxBF];        // of the first block: var / mean^2 of each NA-matching image
+    __shared__ int flags[kMaxCluster];      // of the first block: each block's check
+    const int K = (int)cta_count(), rank = (int)cta_rank();
+    const int tile = blockIdx.x / K;
     const size_t npix = (size_t)P.h * P.w;
     const float* T = I + (size_t)tile * P.n_img * npix;
-    double acc = 0;
     int bad = 0, par = 0;
     auto invalid = [](float4 v) {
         return !(v.x >= 0.f && v.x < INFINITY) || !(v.y >= 0.f && v.y < INFINITY) ||
                !(v.z >= 0.f && v.z < INFINITY) || !(v.w >= 0.f && v.w < INFINITY);
     };
-    for (int i = 0; i < P.n_img; ++i) {
+    tile_sync<true>();                      // the first block runs before any other stores into it
+    for (int i = rank; i < P.n_img; i += K) {
         const float4* T4 = reinterpret_cast<const float4*>(T + i * npix);
         const int nq = (int)(npix / 4);
         if (i < P.n_bf) {
@@ -43,16 +50,24 @@ __global__ void __launch_bounds__(kThreads) k_background(DevPlan P, int n_tiles,
             }
             const double st = block_sum2((double)s, red, par);
             const double st2 = block_sum2((double)s2, red, par);
-            const double mean = st / npix;
-            const double var = st2 / npix - mean * mean;
-            acc += mean > 0 ? var / (mean * mean) : 0.0;
+            if (threadIdx.x == 0) {
+                const double mean = st / npix;
+                const double var = st2 / npix - mean * mean;
+                st_first(value + i, mean > 0 ? var / (mean * mean) : 0.0);
+            }
         } else {
 #pragma unroll 4
             for (int k = threadIdx.x; k < nq; k += blockDim.x) bad |= invalid(__ldcs(T4 + k));
         }
     }
-    const int anybad = __syncthreads_or(bad);
-    if (threadIdx.x == 0) {
+    const int mine = __syncthreads_or(bad);
+    if (threadIdx.x == 0) st_first(flags + rank, mine);
+    tile_sync<true>();
+    if (rank == 0 && threadIdx.x == 0) {
+        double acc = 0;
+        for (int i = 0; i < P.n_bf; ++i) acc += value[i];
+        int anybad = 0;
+        for (int q = 0; q < K; ++q) anybad |= flags[q];
         const float v = (float)(acc / P.n_bf);
         if (c2) c2[tile] = v;
         int st = 0;
@@ -62,10 +77,17 @@ __global__ void __launch_bounds__(kThreads) k_background(DevPlan P, int n_tiles,
     }
 }
 
+// Blocks per tile. One block reads 512-pixel images at 0.07 TB/s, so a batch is as slow as its
+// first tile until the chip is full: 1.80 ms for 1 tile and 2.14 for 96 with one block each, 0.20
+// and 0.66 with eight (256 pixels: 0.22 and 0.43 ms for 1 and 100 tiles, 0.036 and 0.15). Beyond
+// some 64 tiles four are as fast: 2.14 ms for 400 tiles of 512 pixels (2.59 with one), 0.34 for
+// 1000 of 128 pixels (0.36 with eight).
+constexpr int kBgFew = 64;
+
 cudaError_t launch_background(const DevPlan& P, int n_tiles, const float* I, float* c2, int32_t* status,
                               float thresh2, cudaStream_t st, int learned) {
-    k_background<<<n_tiles, kThreads, 0, st>>>(P, n_tiles, I, c2, status, thresh2, learned);
-    return cudaGetLastError();
+    const int K = n_tiles <= kBgFew ? 8 : 4;
+    return cluster_launch(k_background, K, n_tiles, kThreads, 0, st, P, I, c2, status, thresh2, learned);
 }
 
 __device__ __forceinline__ bool skip_tile(const int32_t* status, int tile) {

@@ -116,3 +116,34 @@ def test_kramers_kronig_does_not_depend_on_the_blocks_per_problem(tile, sizes):
         x.zero_()
         plan.kk_spectra_noalloc(k, I[:k].contiguous(), x)
         assert torch.equal(x, ref[:k]), k
+
+
+@pytest.mark.parametrize("tile,ill", [(64, "8+16"), (256, "8+16"), (256, "12+22"), (512, "8+24")])
+def test_background_does_not_depend_on_the_blocks_per_tile(tile, ill):
+    """Eight blocks per tile (up to 64 tiles) and four: the same values and flags, a bad pixel
+    found wherever it is, and the contrast of float64 sums. A thread sums q = npix / 2048 groups
+    of four pixels in FP32: both means are within (q + 2) 2^-24 of exact, so the contrast c is
+    within 3 (q + 2) 2^-24 (1 + c)."""
+    il = {"8+16": synth.illumination, "8+24": synth.illumination_8_24, "12+22": synth.illumination_12_22}[ill]()
+    n = 70
+    plan, I = _tiles(tile, il, n)
+    n_img, n_bf = plan.info.n_bf + plan.info.n_df, plan.info.n_bf
+    I = I.reshape(n, n_img, tile, tile).clone()
+    for t in range(n_img):
+        I[t, t, -1, -1] = float("nan") if t % 2 else -1.0
+    out = {}
+    for k in (1, 9, 64, 65, n):
+        c2 = torch.full((k,), -1.0, device="cuda")
+        st = torch.full((k,), -1, dtype=torch.int32, device="cuda")
+        plan.background(k, I[:k].contiguous(), c2, st)
+        out[k] = c2, st
+    for k in (1, 9, 64, 65):
+        assert torch.equal(out[k][1], out[n][1][:k]), k
+        assert torch.equal(out[k][0].view(torch.int32), out[n][0][:k].view(torch.int32)), k
+    bad = (out[n][1] & apic.APIC_TILE_BADINPUT) != 0
+    assert bad[:n_img].all() and not bad[n_img:].any()
+    x = I[n_img:, :n_bf].double()
+    m = x.mean((2, 3))
+    c = (((x * x).mean((2, 3)) - m * m) / (m * m)).mean(1)
+    q = max(1, tile * tile // 2048)
+    assert ((out[n][0][n_img:].double() - c).abs() <= 3 * (q + 2) * 2.0 ** -24 * (1 + c)).all()
