@@ -472,14 +472,10 @@ apic_status configure(apic_plan* plan) {
     L.grid_syn = sms * std::min(o_syn, o_obj);
     L.grid_sim = sms * o_sim;
     // register-transform synthesis for output sides 512 and 1024 (the Stockham kernel otherwise)
-    L.grid_synr = 0;
     L.smem_synr = synr_smem_bytes(D.H);
-    if (!legacy && (D.H == 512 || D.H == 1024)) {
-        const int o_sr = configure_synr(D.H, L.smem_synr);
-        if (o_sr > 0)
-            L.grid_synr = sms * o_sr;
-        else
-            cudaGetLastError();
+    for (int i = 0; i < 4; ++i) {
+        L.synr_slots[i] = !legacy && (D.H == 512 || D.H == 1024) ? configure_synr(D.H, L.smem_synr, 1 << i) : 0;
+        cudaGetLastError();
     }
     return APIC_OK;
 }

@@ -97,7 +97,8 @@ struct DevPlan {
 struct Launch {
     int grid_kk, grid_ab, grid_df, grid_syn, grid_sim;
     size_t smem_kk, smem_df, smem_syn, smem_sim;
-    int grid_synr;                   // register-transform synthesis (output sides 512, 1024), 0: not used
+    int synr_slots[4];               // register-transform synthesis (output sides 512, 1024): tiles at once with
+                                     // 1, 2, 4, 8 blocks each; 0: not used
     size_t smem_synr;
 };
 
@@ -133,9 +134,9 @@ cudaError_t launch_darkfield(const DevPlan& P, const Launch& L, int n_tiles, con
 cudaError_t launch_synthesize(const DevPlan& P, const Launch& L, int n_tiles, const float2* spec, float2* field,
                               const int32_t* status, cudaStream_t st);
 // Register-transform synthesis for output side H = 32 B (B in 16, 32): dynamic shared memory
-// and blocks per SM (0: unsupported side or failure).
+// and tiles at once with K blocks each (0: unsupported side or failure).
 size_t synr_smem_bytes(int H);
-int configure_synr(int H, size_t smem);
+int configure_synr(int H, size_t smem, int K);
 cudaError_t launch_pupil(const DevPlan& P, int n_tiles, const float* phi, float2* pupil, const int32_t* status,
                          cudaStream_t st);
 cudaError_t launch_sim(const DevPlan& P, const Launch& L, int n_tiles, const float2* obj, const float* phi,

@@ -3,6 +3,7 @@
 #include <math.h>
 
 #include "../../include/apic.h"
+#include "cluster.cuh"
 #include "passes.cuh"
 #include "regfft.cuh"
 
@@ -84,7 +85,9 @@ size_t synr_smem_bytes(int H) {
     return (size_t)kSRWarps * 32 * kSRLd * sizeof(float2) + (size_t)H * sizeof(float2);
 }
 
-template <int B>
+// CL: a cluster of K blocks per tile, the column chunks and the rows dealt over its blocks
+// (same results).
+template <int B, bool CL>
 __global__ void __launch_bounds__(kSRWarps * 32, 1)
 k_synth_reg(DevPlan P, int n_tiles, const float2* __restrict__ spec, float2* __restrict__ field,
             const int32_t* __restrict__ status) {
@@ -101,15 +104,17 @@ k_synth_reg(DevPlan P, int n_tiles, const float2* __restrict__ spec, float2* __r
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float2* hs = areas + warp * 32 * kSRLd;
     const int x0 = P.ap_x0, nbx = P.ap_x1 - P.ap_x0 + 1;
-    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    const int K = CL ? (int)cta_count() : 1, rank = CL ? (int)cta_rank() : 0;
+    for (int tile = blockIdx.x / K; tile < n_tiles; tile += gridDim.x / K) {
         float2* F = field + (size_t)tile * N * N;
         if (status && (status[tile] & (APIC_TILE_BACKGROUND | APIC_TILE_BADINPUT))) {
-            for (size_t t = threadIdx.x; t < (size_t)N * N; t += blockDim.x) F[t] = make_float2(0.f, 0.f);
+            for (size_t t = rank * blockDim.x + threadIdx.x; t < (size_t)N * N; t += K * blockDim.x)
+                F[t] = make_float2(0.f, 0.f);
             continue;
         }
         const float2* sp = spec + (size_t)tile * P.nap;
         // 1: aperture columns, 16 at a time
-        for (int c0 = 0; c0 < nbx; c0 += kSRWarps) {
+        for (int c0 = rank * kSRWarps; c0 < nbx; c0 += K * kSRWarps) {
             const int c = c0 + warp;
             float2 o[32];
             if (c < nbx) {
@@ -143,15 +148,16 @@ k_synth_reg(DevPlan P, int n_tiles, const float2* __restrict__ spec, float2* __r
             }
             __syncthreads();                            // stage consumed before the areas are reused
         }
+        if constexpr (CL) tile_sync<true>();
         // 2: rows (each warp reads its own rows' aperture columns before overwriting them)
-        for (int y = warp; y < N; y += kSRWarps) {
+        for (int y = rank * kSRWarps + warp; y < N; y += K * kSRWarps) {
             float2* row = F + (size_t)y * N;
             float2 v[B], o[32];
 #pragma unroll
             for (int j = 0; j < B; ++j) {
                 const int x = lane + 32 * j;
                 const int c = (x < N / 2 ? x : x - N) - x0;
-                v[j] = (unsigned)c < (unsigned)nbx ? row[c] : make_float2(0.f, 0.f);
+                v[j] = (unsigned)c < (unsigned)nbx ? ldx<CL>(row + c) : make_float2(0.f, 0.f);
             }
             warp_fft_inv<B>(v, o, hs, tw, lane);
             if (lane < B) {
@@ -163,31 +169,44 @@ k_synth_reg(DevPlan P, int n_tiles, const float2* __restrict__ spec, float2* __r
     }
 }
 
-template <int B>
-static int configure_synr_b(size_t smem) {
-    if (raise_smem_limit((const void*)k_synth_reg<B>, smem) != cudaSuccess) return 0;
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_synth_reg<B>, kSRWarps * 32, smem) != cudaSuccess)
-        return 0;
-    return occ;
+using SynKernel = void (*)(DevPlan, int, const float2*, float2*, const int32_t*);
+
+static SynKernel syn_kernel(int H, int K) {
+    if (H == 512) return K > 1 ? k_synth_reg<16, true> : k_synth_reg<16, false>;
+    if (H == 1024) return K > 1 ? k_synth_reg<32, true> : k_synth_reg<32, false>;
+    return nullptr;
 }
 
-int configure_synr(int H, size_t smem) {
-    if (H == 512) return configure_synr_b<16>(smem);
-    if (H == 1024) return configure_synr_b<32>(smem);
-    return 0;
+// Tiles (blocks, or clusters of K blocks) that run at once, 0 on error.
+int configure_synr(int H, size_t smem, int K) {
+    return cluster_slots((const void*)syn_kernel(H, K), kSRWarps * 32, smem, K);
+}
+
+// Blocks per tile with the register transforms: a round of tiles with 1, 2, 4, 8 blocks each
+// takes 513, 261, 139, 81 us at 1024 x 1024 and 154, 85, 50, 29 us at 512 x 512; the fewest
+// rounds times that (one row of figures, between the two, is enough to order them).
+static int synr_cluster(const Launch& L, int n_tiles) {
+    static const int kRound[4] = {100, 53, 30, 17};
+    int best = 0;
+    long least = 0;
+    for (int i = 0; i < 4; ++i) {
+        if (L.synr_slots[i] < 1) continue;
+        const long t = (long)((n_tiles + L.synr_slots[i] - 1) / L.synr_slots[i]) * kRound[i];
+        if (!least || t < least) {
+            least = t;
+            best = i;
+        }
+    }
+    return best;
 }
 
 cudaError_t launch_synthesize(const DevPlan& P, const Launch& L, int n_tiles, const float2* spec, float2* field,
                               const int32_t* status, cudaStream_t st) {
-    if (L.grid_synr > 0 && (P.H == 512 || P.H == 1024)) {
-        const int grid = min(L.grid_synr, n_tiles);
-        if (grid < 1) return cudaSuccess;
-        if (P.H == 512)
-            k_synth_reg<16><<<grid, kSRWarps * 32, L.smem_synr, st>>>(P, n_tiles, spec, field, status);
-        else
-            k_synth_reg<32><<<grid, kSRWarps * 32, L.smem_synr, st>>>(P, n_tiles, spec, field, status);
-        return cudaGetLastError();
+    if (n_tiles < 1) return cudaSuccess;
+    if (L.synr_slots[0] > 0) {
+        const int i = synr_cluster(L, n_tiles), K = 1 << i;
+        return cluster_launch(syn_kernel(P.H, K), K, min(L.synr_slots[i], n_tiles), kSRWarps * 32, L.smem_synr, st, P,
+                              n_tiles, spec, field, status);
     }
     const int grid = min(L.grid_syn, n_tiles);
     k_synthesize<<<grid, kThreads, L.smem_syn, st>>>(P, n_tiles, spec, field, status);

@@ -147,3 +147,24 @@ def test_background_does_not_depend_on_the_blocks_per_tile(tile, ill):
     c = (((x * x).mean((2, 3)) - m * m) / (m * m)).mean(1)
     q = max(1, tile * tile // 2048)
     assert ((out[n][0][n_img:].double() - c).abs() <= 3 * (q + 2) * 2.0 ** -24 * (1 + c)).all()
+
+
+@pytest.mark.parametrize("tile,up,sizes", [(256, 2, (1, 16, 30, 60, 152, 200)), (512, 2, (1, 16, 30, 60, 152, 200)),
+                                           (128, 2, (1, 3))])
+def test_synthesis_does_not_depend_on_the_blocks_per_tile(tile, up, sizes):
+    """Eight blocks per tile down to one: the same fields."""
+    ill = synth.illumination()
+    n = max(sizes)
+    plan = apic.Plan.from_illumination(tile, ill, max_tiles=n, upsample=up)
+    H, nap = plan.info.out_h, plan.info.n_aperture
+    g = torch.Generator(device="cuda").manual_seed(1)
+    spec = torch.randn((n, nap, 2), generator=g, device="cuda")
+    ref = torch.empty((n, H, 2 * H), device="cuda")
+    plan.synthesize(n, spec, ref)
+    for k in sizes:
+        f = torch.full((k, H, 2 * H), 7.0, device="cuda")
+        plan.synthesize(k, spec[:k].contiguous(), f)
+        assert torch.equal(f, ref[:k]), k
+    # Parseval: the field's energy is the spectrum's, up to the transform's scale, for every tile alike
+    e = ref.double().square().sum((1, 2)) / spec.double().square().sum((1, 2))
+    assert float((e / e[0] - 1).abs().max()) < 1e-5
