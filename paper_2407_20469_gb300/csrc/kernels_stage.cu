@@ -230,34 +230,97 @@ cudaError_t launch_kk_grid(const DevPlan& P, int grid, size_t smem, int n_tiles,
 // stage 2 runs `passes` refinements on the rows of Eq. 10. Products are
 // accumulated per thread in FP32, summed across the block in FP64, and the
 // 12 x 12 normal equations are solved in FP64 with the plan's Cholesky factors.
-__device__ void reduce12(float* g, double* red, double* out) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int z = 0; z < 12; ++z) {
-        double v = g[z];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) red[warp * 12 + z] = v;
+// CL: the tile's 512 threads spread over a cluster of K blocks of 512 / K threads; the warps' sums go
+// to every block, and each adds them in warp order and solves, so K does not change the result.
+// Bound by the latency of the rows' loads and, per sum, of the FP64 pipe: a call on one tile of
+// 128, 256 and 512 pixels takes 0.041, 0.088 and 0.28 ms, against 0.12, 0.20 and 0.51 with one block,
+// two rows in flight, each value summed over all lanes and one thread solving.
+constexpr int kAbWarps = kThreads / 32;
+
+struct AbShared {
+    double s12[2][kAbWarps * 12], s1[2][kAbWarps];      // warps' sums, two sets in turn: a block of a
+                                                        // cluster may be one sum ahead of another
+    double L[2][144], rd[2][12];                        // factors of the two stages, 1 / their diagonals
+    double cc[12], cbest[12];
+    float cf[12];
+};
+
+// p[0] = v in every block of the tile
+template <bool CL>
+__device__ __forceinline__ void st_all(double* p, double v) {
+    if constexpr (!CL) {
+        *p = v;
+    } else {
+        const uint32_t a = (uint32_t)__cvta_generic_to_shared(p), K = cta_count();
+        for (uint32_t q = 0; q < K; ++q) {
+            uint32_t ra;
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(q));
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"(v) : "memory");
+        }
     }
-    __syncthreads();
-    if (threadIdx.x < 12) {
-        double t = 0;
-        for (int w = 0; w < nw; ++w) t += red[w * 12 + threadIdx.x];
-        out[threadIdx.x] = t;
-    }
-    __syncthreads();
 }
 
-__device__ void chol_solve12(const double* L, const double* b, double* x) {
-    double y[12];
-    for (int i = 0; i < 12; ++i) {
-        double s = b[i];
-        for (int k = 0; k < i; ++k) s -= L[i * 12 + k] * y[k];
-        y[i] = s / L[i * 12 + i];
+// Solution of L L^T x = b by the lanes of a warp, lane i < 12 with b_i in and x_i out: as each
+// unknown is found, the lanes of those to come take its term off. rd: 1 / L_ii.
+__device__ __forceinline__ double chol_solve12(const double* L, const double* rd, double b) {
+    const int lane = threadIdx.x & 31;
+    double y = b;
+    for (int j = 0; j < 12; ++j) {
+        const double yj = __shfl_sync(0xffffffffu, y, j) * rd[j];
+        if (lane == j) y = yj;
+        if (lane > j && lane < 12) y -= L[lane * 12 + j] * yj;
     }
-    for (int i = 11; i >= 0; --i) {
-        double s = y[i];
-        for (int k = i + 1; k < 12; ++k) s -= L[k * 12 + i] * x[k];
-        x[i] = s / L[i * 12 + i];
+    for (int j = 11; j >= 0; --j) {
+        const double xj = __shfl_sync(0xffffffffu, y, j) * rd[j];
+        if (lane == j) y = xj;
+        if (lane < j) y -= L[j * 12 + lane] * xj;
     }
+    return y;
+}
+
+// Sum of the tile's g[12] (FP64 from here on), then cc = (add ? cc : 0) + the solution of
+// stage `which`, cf = cc in FP32. The warp's sum halves the values with the lanes (13 FP64 adds a
+// lane where a sum of each value over all lanes takes 60; the FP64 pipe adds 2 a clock and SM).
+template <bool CL>
+__device__ void sum_solve12(const float (&g)[12], AbShared& S, int& turn, int vt, int which, bool add) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4, h2 = lane & 2;
+    double a[6], b[3], c[2];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        const float other = __shfl_xor_sync(kAll, h16 ? g[i] : g[6 + i], 16);
+        a[i] = (double)(h16 ? g[6 + i] : g[i]) + (double)other;
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const double other = __shfl_xor_sync(kAll, h8 ? a[i] : a[3 + i], 8);
+        b[i] = (h8 ? a[3 + i] : a[i]) + other;
+    }
+    {
+        const double o0 = __shfl_xor_sync(kAll, h4 ? b[0] : b[2], 4), o1 = __shfl_xor_sync(kAll, b[1], 4);
+        c[0] = (h4 ? b[2] : b[0]) + o0;                 // value 2 or 0
+        c[1] = b[1] + o1;
+    }
+    double d = (h2 ? c[1] : c[0]) + __shfl_xor_sync(kAll, h2 ? c[0] : c[1], 2);
+    d += __shfl_xor_sync(kAll, d, 1);
+    // lanes with both bits of (4, 2) set hold value 1 once more
+    if (!(lane & 1) && !(h4 && h2))
+        st_all<CL>(S.s12[turn] + (vt >> 5) * 12 + 6 * h16 + 3 * h8 + (h2 ? 1 : h4 ? 2 : 0), d);
+    tile_sync<CL>();
+    if (threadIdx.x < 32) {
+        const int i = min(lane, 11);
+        double t = 0;
+        for (int w = 0; w < kAbWarps; ++w) t += S.s12[turn][w * 12 + i];
+        const double x = chol_solve12(S.L[which], S.rd[which], t);
+        if (lane < 12) {
+            const double v = add ? S.cc[lane] + x : x;
+            S.cc[lane] = v;
+            S.cf[lane] = (float)v;
+        }
+    }
+    turn ^= 1;
+    __syncthreads();
 }
 
 // The 12 basis differences of row r: three 16-byte loads (scalar loads of a 48-byte row by
@@ -279,123 +342,133 @@ struct Row12 {
 };
 
 // Refinement passes c <- c + LS(wrap(beta - D c)) from the coefficients in
-// cc / cf (shared); returns the sum of squared wrapped residuals of the rows
-// at the final coefficients (every thread gets it).
-__device__ double value_passes(const DevPlan& P, const float* beta, int passes, double* cc, float* cf, double* dc,
-                               double* rhs, double* red) {
-    float g[12];
+// cc / cf (shared).
+template <bool CL>
+__device__ void value_passes(const DevPlan& P, const float* beta, int passes, AbShared& S, int& turn, int vt) {
     for (int pass = 0; pass < passes; ++pass) {
+        float g[12];
         for (int z = 0; z < 12; ++z) g[z] = 0.f;
-#pragma unroll 2
-        for (int r = threadIdx.x; r < P.nrows; r += blockDim.x) {
+#pragma unroll (CL ? 4 : 2)
+        for (int r = vt; r < P.nrows; r += kThreads) {
             const Row12 A(P.row_A, r);
             float pred = 0.f;
-            for (int z = 0; z < 12; ++z) pred += A[z] * cf[z];
+            for (int z = 0; z < 12; ++z) pred += A[z] * S.cf[z];
             const float e = wrap_pi(beta[r] - pred);
             for (int z = 0; z < 12; ++z) g[z] += A[z] * e;
         }
-        reduce12(g, red, rhs);
-        if (threadIdx.x == 0) {
-            chol_solve12(P.Lval, rhs, dc);
-            for (int z = 0; z < 12; ++z) {
-                cc[z] += dc[z];
-                cf[z] = (float)cc[z];
-            }
-        }
-        __syncthreads();
+        sum_solve12<CL>(g, S, turn, vt, 1, true);
     }
+}
+
+// Sum of the squared wrapped residuals of cf, in every thread.
+template <bool CL>
+__device__ double value_residual(const DevPlan& P, const float* beta, AbShared& S, int& turn, int vt) {
     double res = 0;
-#pragma unroll 2
-    for (int r = threadIdx.x; r < P.nrows; r += blockDim.x) {
+#pragma unroll (CL ? 4 : 2)
+    for (int r = vt; r < P.nrows; r += kThreads) {
         const Row12 A(P.row_A, r);
         float pred = 0.f;
-        for (int z = 0; z < 12; ++z) pred += A[z] * cf[z];
+        for (int z = 0; z < 12; ++z) pred += A[z] * S.cf[z];
         const float e = wrap_pi(beta[r] - pred);
         res += (double)(e * e);
     }
-    return block_sum(res, red);
+    for (int o = 16; o > 0; o >>= 1) res += __shfl_xor_sync(0xffffffffu, res, o);
+    if ((threadIdx.x & 31) == 0) st_all<CL>(S.s1[turn] + (vt >> 5), res);
+    tile_sync<CL>();
+    double t = 0;
+    for (int w = 0; w < kAbWarps; ++w) t += S.s1[turn][w];
+    turn ^= 1;
+    return t;
 }
 
 // c0 [tiles][15] (may be NULL): learned coefficients. Tiles marked
 // APIC_TILE_LEARNED take c0 as their result. With `warm`, every solved tile
 // also runs the refinement passes from c0 and keeps whichever of the two
 // solutions leaves the smaller wrapped residual (then sets APIC_TILE_WARM).
-__global__ void __launch_bounds__(kThreads) k_aberration(DevPlan P, int n_tiles, const float2* __restrict__ xdisc,
-                                                         float* __restrict__ zern, float* __restrict__ beta_scratch,
-                                                         int passes, int32_t* __restrict__ status,
-                                                         const float* __restrict__ c0, int warm) {
-    __shared__ double red[16 * 12];
-    __shared__ double rhs[12], cc[12], dc[12], cbest[12];
-    __shared__ float cf[12];
-    float* beta = beta_scratch + (size_t)blockIdx.x * P.nrows;
-    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+template <bool CL>
+__global__ void __launch_bounds__(kThreads, CL ? 1 : 2)
+k_aberration(DevPlan P, int n_tiles, const float2* __restrict__ xdisc, float* __restrict__ zern,
+             float* __restrict__ beta_scratch, int passes, int32_t* __restrict__ status,
+             const float* __restrict__ c0, int warm) {
+    __shared__ AbShared S;
+    const int K = CL ? (int)cta_count() : 1, rank = CL ? (int)cta_rank() : 0;
+    const int vt = rank * blockDim.x + threadIdx.x;         // of the tile's 512 threads
+    float* beta = beta_scratch + (size_t)(blockIdx.x / K) * P.nrows;
+    int turn = 0;
+    for (int i = threadIdx.x; i < 288; i += blockDim.x) (&S.L[0][0])[i] = i < 144 ? P.Lgrad[i] : P.Lval[i - 144];
+    if (threadIdx.x < 24) {
+        const int w = threadIdx.x / 12, i = threadIdx.x - 12 * w;
+        S.rd[w][i] = 1.0 / (w ? P.Lval : P.Lgrad)[i * 13];
+    }
+    tile_sync<CL>();                                        // and every block runs before any stores into it
+    for (int tile = blockIdx.x / K; tile < n_tiles; tile += gridDim.x / K) {
+        float* Z = zern + (size_t)tile * APIC_N_ZERNIKE;
         if (skip_tile(status, tile)) {
-            if (threadIdx.x < APIC_N_ZERNIKE) zern[(size_t)tile * APIC_N_ZERNIKE + threadIdx.x] = 0.f;
+            if (vt < APIC_N_ZERNIKE) Z[vt] = 0.f;
             continue;
         }
         if (c0 && status && (status[tile] & APIC_TILE_LEARNED)) {
-            if (threadIdx.x < APIC_N_ZERNIKE)
-                zern[(size_t)tile * APIC_N_ZERNIKE + threadIdx.x] =
-                    threadIdx.x < 3 ? 0.f : c0[(size_t)tile * APIC_N_ZERNIKE + threadIdx.x];
+            if (vt < APIC_N_ZERNIKE) Z[vt] = vt < 3 ? 0.f : c0[(size_t)tile * APIC_N_ZERNIKE + vt];
             continue;
         }
         const float2* X = xdisc + (size_t)tile * P.n_bf * P.npup;
-        for (int r = threadIdx.x; r < P.nrows; r += blockDim.x) {
-            const int il = P.row_il[r];
-            const float2 a = X[(size_t)(il & 0xffff) * P.npup + P.row_pi[r]];
-            const float2 b = X[(size_t)(il >> 16) * P.npup + P.row_pl[r]];
+#pragma unroll 4
+        for (int r = vt; r < P.nrows; r += kThreads) {
+            const int il = __ldg(P.row_il + r);
+            const float2 a = __ldg(X + (size_t)(il & 0xffff) * P.npup + __ldg(P.row_pi + r));
+            const float2 b = __ldg(X + (size_t)(il >> 16) * P.npup + __ldg(P.row_pl + r));
             const float2 z = cmulc(a, b);
             beta[r] = atan2f(z.y, z.x);
         }
-        __syncthreads();
+        tile_sync<CL>();
         float g[12];
         for (int z = 0; z < 12; ++z) g[z] = 0.f;
-        for (int r = threadIdx.x; r < P.nrows; r += blockDim.x) {
+#pragma unroll (CL ? 2 : 1)
+        for (int r = vt; r < P.nrows; r += kThreads) {
             const Row12 A(P.row_A, r);
             const float br = beta[r];
-            const int nb[2] = {P.row_nx[r], P.row_ny[r]};
-            for (int d = 0; d < 2; ++d) {
-                if (nb[d] < 0) continue;
-                const Row12 A2(P.row_A, nb[d]);
-                const float e = wrap_pi(beta[nb[d]] - br);
-                for (int z = 0; z < 12; ++z) g[z] += (A2[z] - A[z]) * e;
+            const int nx = __ldg(P.row_nx + r), ny = __ldg(P.row_ny + r);
+            const int jx = nx < 0 ? r : nx, jy = ny < 0 ? r : ny;
+            const Row12 Ax(P.row_A, jx), Ay(P.row_A, jy);
+            const float ex = wrap_pi(ldx<CL>(beta + jx) - br), ey = wrap_pi(ldx<CL>(beta + jy) - br);
+            for (int z = 0; z < 12; ++z) {
+                if (nx >= 0) g[z] += (Ax[z] - A[z]) * ex;
+                if (ny >= 0) g[z] += (Ay[z] - A[z]) * ey;
             }
         }
-        reduce12(g, red, rhs);
-        if (threadIdx.x == 0) {
-            chol_solve12(P.Lgrad, rhs, cc);
-            for (int z = 0; z < 12; ++z) cf[z] = (float)cc[z];
-        }
-        __syncthreads();
+        sum_solve12<CL>(g, S, turn, vt, 0, false);
+        value_passes<CL>(P, beta, passes, S, turn, vt);
         bool won = false;
         if (c0 && warm) {
-            const double res = value_passes(P, beta, passes, cc, cf, dc, rhs, red);
+            const double res = value_residual<CL>(P, beta, S, turn, vt);
             if (threadIdx.x < 12) {
-                cbest[threadIdx.x] = cc[threadIdx.x];
-                cc[threadIdx.x] = c0[(size_t)tile * APIC_N_ZERNIKE + 3 + threadIdx.x];
-                cf[threadIdx.x] = (float)cc[threadIdx.x];
+                S.cbest[threadIdx.x] = S.cc[threadIdx.x];
+                S.cc[threadIdx.x] = c0[(size_t)tile * APIC_N_ZERNIKE + 3 + threadIdx.x];
+                S.cf[threadIdx.x] = (float)S.cc[threadIdx.x];
             }
             __syncthreads();
-            const double res_w = value_passes(P, beta, passes, cc, cf, dc, rhs, red);
+            value_passes<CL>(P, beta, passes, S, turn, vt);
+            const double res_w = value_residual<CL>(P, beta, S, turn, vt);
             won = res_w < res;
-            if (!won && threadIdx.x < 12) cc[threadIdx.x] = cbest[threadIdx.x];
+            if (!won && threadIdx.x < 12) S.cc[threadIdx.x] = S.cbest[threadIdx.x];
             __syncthreads();
-        } else {
-            value_passes(P, beta, passes, cc, cf, dc, rhs, red);
         }
-        if (threadIdx.x < APIC_N_ZERNIKE)
-            zern[(size_t)tile * APIC_N_ZERNIKE + threadIdx.x] = threadIdx.x < 3 ? 0.f : (float)cc[threadIdx.x - 3];
-        if (won && status && threadIdx.x == 0) status[tile] |= APIC_TILE_WARM;
-        __syncthreads();
+        if (vt < APIC_N_ZERNIKE) Z[vt] = vt < 3 ? 0.f : (float)S.cc[vt - 3];
+        if (won && status && vt == 0) status[tile] |= APIC_TILE_WARM;
+        tile_sync<CL>();                                    // cc and beta are overwritten for the next tile
     }
 }
 
+// Two blocks per tile while they all run at once (512 pixels, 8 + 24: 0.41 -> 0.28 ms for 1 tile,
+// 0.65 -> 0.53 for 152; 304 tiles would take 1.03 instead of 0.79). Four or eight gain nothing
+// more (0.26 ms for 1 tile): a thread's rows are then what a tile waits for.
 cudaError_t launch_aberration(const DevPlan& P, const Launch& L, int n_tiles, const float2* xdisc, float* zern,
                               float* beta_scratch, int passes, int32_t* status, cudaStream_t st, const float* c0,
                               int warm) {
-    const int grid = min(L.grid_ab, n_tiles);
-    k_aberration<<<grid, kThreads, 0, st>>>(P, n_tiles, xdisc, zern, beta_scratch, passes, status, c0, warm);
-    return cudaGetLastError();
+    const int slots = min(L.grid_ab, n_tiles);
+    const int K = 2 * slots <= L.grid_ab ? 2 : 1;
+    return cluster_launch(K > 1 ? k_aberration<true> : k_aberration<false>, K, slots, kThreads / K, 0, st, P, n_tiles,
+                          xdisc, zern, beta_scratch, passes, status, c0, warm);
 }
 
 // ---------------------------------------------------------------- phase table
@@ -491,7 +564,7 @@ int configure_kernel(int which, size_t smem) {
     const void* f = nullptr;
     switch (which) {
         case 0: f = (const void*)k_kk; break;
-        case 1: f = (const void*)k_aberration; break;
+        case 1: f = (const void*)k_aberration<false>; break;
         case 2: f = (const void*)k_darkfield; break;
         case 3: f = (const void*)k_synthesize; break;
         case 4: f = (const void*)k_sim_images; break;

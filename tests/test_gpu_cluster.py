@@ -168,3 +168,22 @@ def test_synthesis_does_not_depend_on_the_blocks_per_tile(tile, up, sizes):
     # Parseval: the field's energy is the spectrum's, up to the transform's scale, for every tile alike
     e = ref.double().square().sum((1, 2)) / spec.double().square().sum((1, 2))
     assert float((e / e[0] - 1).abs().max()) < 1e-5
+
+
+@pytest.mark.parametrize("tile,ill", [(64, "8+16"), (128, "12+22"), (256, "8+16")])
+def test_aberration_does_not_depend_on_the_blocks_per_tile(tile, ill):
+    """Two blocks per tile (up to a tile per SM) and one, a batch beyond the resident blocks:
+    the same coefficients."""
+    il = synth.illumination_12_22() if ill == "12+22" else synth.illumination()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 2 * sms + 3
+    plan, I = _tiles(tile, il, n)
+    x = torch.empty((n, plan.info.n_bf, plan.info.n_pupil, 2), device="cuda")
+    plan.kk_spectra(n, I, x)
+    ref = torch.empty((n, 15), device="cuda")
+    plan.aberration(n, x, ref)
+    assert bool(torch.isfinite(ref).all()) and float(ref[:, 3:].abs().max()) > 0.01
+    for k in (1, 20, sms, sms + 1):
+        z = torch.full((k, 15), 7.0, device="cuda")
+        plan.aberration(k, x[:k].contiguous(), z)
+        assert torch.equal(z, ref[:k]), k
