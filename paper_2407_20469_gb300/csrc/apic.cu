@@ -595,18 +595,25 @@ struct DfOption {
     double t;
 };
 
-std::vector<DfOption> df_options(const apic_plan* p) {
+// On the stack, like the rounds: a batch call allocates nothing here.
+struct DfOptions {
+    DfOption o[8];
+    int n = 0;
+};
+
+DfOptions df_options(const apic_plan* p) {
     static const double t128[][2] = {{3, 0.77}, {5, 0.61}, {8, 0.59}};
     static const double t256[][2] = {{3, 0.54}, {4, 0.43}, {6, 0.40}, {8, 0.32}};
     static const double t512[][2] = {{2, 0.58}, {3, 0.42}, {4, 0.37}, {5, 0.31}, {6, 0.29}, {8, 0.27}, {10, 0.22}};
-    std::vector<DfOption> o{{1, p->grid_dfr, 1.0}};
+    DfOptions r;
+    r.o[r.n++] = {1, p->grid_dfr, 1.0};
     auto add = [&](const double (*t)[2], int n) {
         for (int i = 0; i < n; ++i) {
             // clusters that run at once, and that the scratch of one wave holds
             const int K = (int)t[i][0];
             const size_t each = p->dev.mr == 512 ? p->df_per_block : dfc_scratch_bytes(p->dev);
             const int cap = (int)std::min<size_t>(p->df_slots[K], p->df_slots_alloc * p->df_per_block / each);
-            if (cap > 0) o.push_back({K, cap, t[i][1]});
+            if (cap > 0) r.o[r.n++] = {K, cap, t[i][1]};
         }
     };
     switch (p->dev.h) {
@@ -614,28 +621,43 @@ std::vector<DfOption> df_options(const apic_plan* p) {
         case 256: add(t256, 4); break;
         case 512: add(t512, 7); break;
     }
-    return o;
+    return r;
 }
 
 // Rounds for n tiles (less than a full wave): the sequence of options with the least total
-// time, in round times of one block per tile (dynamic programming over the tiles left).
-double df_schedule(const apic_plan* p, int n, std::vector<DfOption>* rounds) {
-    const std::vector<DfOption> opt = df_options(p);
-    std::vector<double> best(n + 1, 0.0);
-    std::vector<int> pick(n + 1, 0);
+// time t, in round times of one block per tile (dynamic programming over the tiles left).
+// One round of one block per tile always serves, so there are at most 1 / 0.22 rounds.
+struct DfRounds {
+    DfOption o[8];
+    int n = 0;
+    double t = 0.0;
+};
+
+DfRounds df_schedule(const apic_plan* p, int n) {
+    constexpr int kMax = 1024;
+    const DfOptions opt = df_options(p);
+    DfRounds r;
+    if (n < 1) return r;
+    if (n > kMax) {
+        r.o[r.n++] = opt.o[0];
+        r.t = 1.0;
+        return r;
+    }
+    double best[kMax + 1] = {0.0};
+    unsigned char pick[kMax + 1] = {0};
     for (int k = 1; k <= n; ++k) {
         best[k] = 1e30;
-        for (int i = 0; i < (int)opt.size(); ++i) {
-            const double t = opt[i].t + best[std::max(0, k - opt[i].cap)];
+        for (int i = 0; i < opt.n; ++i) {
+            const double t = opt.o[i].t + best[std::max(0, k - opt.o[i].cap)];
             if (t < best[k]) {
                 best[k] = t;
-                pick[k] = i;
+                pick[k] = (unsigned char)i;
             }
         }
     }
-    if (rounds)
-        for (int k = n; k > 0; k -= opt[pick[k]].cap) rounds->push_back(opt[pick[k]]);
-    return best[n];
+    for (int k = n; k > 0 && r.n < 8; k -= opt.o[pick[k]].cap) r.o[r.n++] = opt.o[pick[k]];
+    r.t = best[n];
+    return r;
 }
 
 bool df_may_cluster(const apic_plan* p) { return p->use_reg && p->df_rounds && p->df_cluster == 1; }
@@ -653,9 +675,9 @@ cudaError_t launch_df(apic_plan* p, int n_tiles, const float* I, float2* spec, i
         const cudaError_t e = launch_df_on(p, a, I, p->phi, spec, status, false, st);
         if (e != cudaSuccess) return e;
     }
-    std::vector<DfOption> rounds;
-    df_schedule(p, n_tiles - a, &rounds);
-    for (const DfOption& o : rounds) {
+    const DfRounds rounds = df_schedule(p, n_tiles - a);
+    for (int i = 0; i < rounds.n; ++i) {
+        const DfOption& o = rounds.o[i];
         const int k = std::min(o.cap, n_tiles - a);
         const float* Ia = I + (size_t)a * in_tile;
         const float* ph = p->phi + (size_t)a * D.npup;
@@ -684,7 +706,7 @@ cudaError_t launch_df(apic_plan* p, int n_tiles, const float* I, float2* spec, i
 // against 15.6 ms).
 bool df_rounds_beat_split(const apic_plan* p, int r, int m0) {
     constexpr double kPre = 9e-4;
-    return df_may_cluster(p) && df_schedule(p, r, nullptr) + kPre * m0 < 1.0;
+    return df_may_cluster(p) && df_schedule(p, r).t + kPre * m0 < 1.0;
 }
 
 apic_status check_plan(const apic_plan* plan, int n_tiles) {
