@@ -248,14 +248,15 @@ __global__ void k_blend(int rows, int cols, int u, int L, const float2* __restri
     }
 }
 
-// Output pixel pairs (X, X + 1), X even, over a stripe of kBlendRows rows. With u even,
+// Output pixel pairs (X, X + 1), X even, over a stripe of rows (at most kBlendRows). With u even,
 // window edges in output pixels are even, so both pixels of a pair lie in the same windows
 // and their field values are one 16-byte load. The windows covering a pixel along one axis
 // are a contiguous run ending at the last one that starts at or before it; each thread
-// finds its column run and ramps once, and the block's first kBlendRows threads find the
+// finds its column run and ramps once, and the block's first `stripe` threads find the
 // row runs and ramps of the stripe into shared memory. A run longer than kMaxCover falls
 // back to the per-pixel rule.
 constexpr int kMaxCover = 4, kBlendThreads = 128, kBlendRows = 32, kBlendBatch = 4;
+constexpr int kBlendFill = 152 * 64;         // four times the blocks of 128 threads that run at once
 
 // run of windows (starts u * start(0..count-1), increasing) covering p: last index and length
 // (length kMaxCover + 1 when longer than kMaxCover)
@@ -279,13 +280,13 @@ __global__ void __launch_bounds__(kBlendThreads) k_blend_pairs(int rows, int col
                                                                 const float2* __restrict__ field,
                                                                 const int32_t* __restrict__ win,
                                                                 const float2* __restrict__ z, int Ho, int Wo,
-                                                                float2* __restrict__ out) {
+                                                                float2* __restrict__ out, int stripe) {
     __shared__ int s_last[kBlendRows], s_n[kBlendRows], s_sy[kBlendRows][kMaxCover];
     __shared__ float s_wy[kBlendRows][kMaxCover];
-    const int Y0 = blockIdx.y * kBlendRows, Y1 = min(Ho, Y0 + kBlendRows);
+    const int Y0 = blockIdx.y * stripe, Y1 = min(Ho, Y0 + stripe);
     auto ystart = [&](int i) { return win_y(win, cols, i); };
     auto xstart = [&](int j) { return win_x(win, j); };
-    if (threadIdx.x < kBlendRows && Y0 + (int)threadIdx.x < Y1) {
+    if (threadIdx.x < stripe && Y0 + (int)threadIdx.x < Y1) {
         const int r = threadIdx.x, Y = Y0 + r;
         const int2 run = cover_run(ystart, rows, u, L, Y);
         s_last[r] = run.x;
@@ -401,9 +402,15 @@ cudaError_t launch_blend(const DevPlan& P, int n_tiles, int rows, int cols, cons
     const int Ho = u * Hs, Wo = u * Ws;
     const bool pairs = u % 2 == 0 && (((uintptr_t)field | (uintptr_t)out) & 15) == 0;
     if (pairs) {
-        const dim3 grid((unsigned)((Wo / 2 + kBlendThreads - 1) / kBlendThreads),
-                        (unsigned)((Ho + kBlendRows - 1) / kBlendRows));
-        k_blend_pairs<<<grid, kBlendThreads, 0, st>>>(rows, cols, u, L, field, win, z, Ho, Wo, out);
+        // A block takes its rows one after the other, ~1.3 us each: shorter stripes until there
+        // are kBlendFill blocks. The kernel alone, stripes of 32 rows -> this rule: 10 x 11 windows of
+        // 128 57 -> 38 us, 17 x 22 of 128 151 -> 120, 6 x 22 of 256 157 -> 128, 12 x 25 of 256
+        // 254 -> 230; 16 x 32 of 256 keeps 32 rows.
+        const int bx = (Wo / 2 + kBlendThreads - 1) / kBlendThreads;
+        int stripe = kBlendRows;
+        while (stripe > kBlendBatch && (long long)bx * ((Ho + stripe - 1) / stripe) < kBlendFill) stripe /= 2;
+        const dim3 grid((unsigned)bx, (unsigned)((Ho + stripe - 1) / stripe));
+        k_blend_pairs<<<grid, kBlendThreads, 0, st>>>(rows, cols, u, L, field, win, z, Ho, Wo, out, stripe);
     } else {
         k_blend<<<grid_for((size_t)Ho * Wo), 256, 0, st>>>(rows, cols, u, L, field, win, z, Ho, Wo, out);
     }

@@ -205,3 +205,29 @@ def test_skipped_background_tiles_leave_the_others_bit_exact(n):
     assert np.all((st[blank] & apic.APIC_TILE_BACKGROUND) != 0) and np.all(st[~blank] == 0)
     assert torch.count_nonzero(f_mix[torch.as_tensor(np.nonzero(blank)[0], device="cuda")]) == 0
     assert torch.equal(f_mix[idx], f_s) and torch.equal(z_mix[idx], z_s)
+
+
+@pytest.mark.parametrize("rows,cols,stride", [(2, 3, 59), (9, 11, 62), (13, 20, 61), (25, 25, 59), (38, 39, 61)])
+def test_blend_of_crops_of_one_image_is_the_image(rows, cols, stride):
+    """Windows cut from one image, so every phase is 0 and every weighted mean is the pixel, for
+    stripes of 4, 8, 16 and 32 rows per block and ragged last stripes. FP32: a step of the phase
+    chain is off by at most a rounding of the correlation's terms, 2^-24, a chain has rows + cols
+    steps, a weighted mean some ten roundings."""
+    t, u = 64, 2
+    plan = apic.Plan.from_illumination(t, synth.illumination(), max_tiles=1)
+    Hs, Ws = t + (rows - 1) * stride, t + (cols - 1) * stride
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    F = torch.polar(0.5 + torch.rand((u * Hs, u * Ws), generator=g, device="cuda"),
+                    6.0 * torch.rand((u * Hs, u * Ws), generator=g, device="cuda"))
+    L, n = u * t, rows * cols
+    f = torch.stack([F[u * stride * i:u * stride * i + L, u * stride * j:u * stride * j + L]
+                     for i in range(rows) for j in range(cols)])
+    win = torch.zeros((n, 6), dtype=torch.int32)
+    win[:, 0] = torch.arange(n) // cols * stride
+    win[:, 1] = torch.arange(n) % cols * stride
+    corr = torch.empty((n, 2, 2), device="cuda")
+    phase = torch.empty((n, 2), device="cuda")
+    out = torch.full((u * Hs, u * Ws, 2), 9.0, device="cuda")
+    plan.blend_fields(n, torch.view_as_real(f).contiguous(), win.cuda(), rows, cols, Hs, Ws, corr, phase, out)
+    err = (torch.view_as_complex(out) - F).abs() / F.abs()
+    assert float(err.max()) <= (rows + cols + 10) * 2.0 ** -24 * 2
