@@ -53,8 +53,8 @@ WORKLOADS = {
 PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 PROFILES = os.path.join(ROOT, "profiles")
 DEFAULT_DF_TOL = 3e-4          # the library's darkfield CG tolerance (apic_params.df_tol <= 0)
-DF_SOURCES = {256: ["kernels_dfr.cu", "regfft.cuh", "common.cuh", "internal.cuh"],
-              512: ["kernels_dfw.cu", "regfft.cuh", "t4grid.cuh", "common.cuh", "internal.cuh"]}
+DF_SOURCES = {256: ["kernels_dfr.cu", "regfft.cuh", "t4grid.cuh", "tmem.cuh", "common.cuh"],
+              512: ["kernels_dfw.cu", "regfft.cuh", "t4grid.cuh", "rowsum.cuh", "cluster.cuh", "common.cuh"]}
 DF_KERNEL = {256: "k_darkfield_reg", 512: "k_darkfield_wide"}
 HOST_E2E_RAM_FRAC = 0.45       # pinned host buffers of the end-to-end leg: at most this share of host RAM
 
@@ -694,7 +694,7 @@ def gpu_arm(args):
                    "launch": "direct C-ABI calls", "tiles_per_s": world * T * args.steps / (ms / 1e3),
                    "df_tol": args.df_tol or "library default", "fft_m": info.fft_m,
                    "precision": "FFTs, elementwise math and CG vectors FP32; aberration normal equations and "
-                                "darkfield CG step lengths / cross-warp sums FP64",
+                                "darkfield CG step lengths / cross-warp sums FP64 (float pairs at 512 pixels)",
                    "tiles_status_nonzero": int(np.count_nonzero(status_np))},
         "roofline": roofline, "e2e": e2e, "gpu_launches": cnt["launches"], "clocks": clk,
     }

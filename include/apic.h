@@ -343,8 +343,8 @@ apic_status apic_stitch(apic_plan* plan, int n_tiles, const float* d_xdisc,
 
 /*
  * Darkfield extension (Eq. 11-13), darkfield images in plan order, each solved
- * by CGLS on C U = b with FFT correlations (FP32 transforms, FP64 scalars and
- * solution accumulation). Updates d_spec in place; ORs APIC_TILE_NOTCONV into
+ * by CGLS on C U = b with FFT correlations (FP32 transforms, FP64 scalars -
+ * float pairs at 512 pixels - and solution accumulation). Updates d_spec in place; ORs APIC_TILE_NOTCONV into
  * d_tile_status (may be NULL) where a solve ended above its tolerance.
  */
 apic_status apic_darkfield(apic_plan* plan, int n_tiles, const float* d_intensity,
