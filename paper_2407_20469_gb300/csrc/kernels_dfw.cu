@@ -443,11 +443,14 @@ __device__ __noinline__ void wpass_image_rows(HWw w, const float2* tw, const flo
 //   [0, setup)        during an image's setup: half-warp areas of the 512-point
 //                     transforms (17 x 32 values each), or the 32-column image
 //                     stage, or the output stage of the image columns
-//   [tw, tw_end)      step twiddles of the camera grid and of the image's row and
-//                     column grids
-//   [red, total)      two lists of the U rows' sums
+//   [tw, total)       step twiddles of the camera grid and of the image's row and
+//                     column grids. The camera grid's serve an image's setup alone and are
+//                     made anew for each image; during the CG two lists of the U rows' sums
+//                     take their place. (Beside them the lists took 2 KB, and plans whose CG
+//                     vectors fill the block lost this kernel: 3967 unknowns fit, 3902 did
+//                     then; 8 + 16 images on rings at NA 0.29 and 0.376 have 3933.)
 struct DFWSmem {
-    size_t vec, tw, red, total;
+    size_t vec, tw, total;
 };
 
 __host__ __device__ inline size_t walign16(size_t b) { return (b + 15) & ~(size_t)15; }
@@ -462,8 +465,7 @@ __host__ __device__ inline DFWSmem dfw_smem_layout(int max_N, int band) {
     const size_t stage_f = (size_t)16 * kWBN * kWStageLd * sizeof(float);
     const size_t setup = std::max(setup_hw, std::max(stage_c, stage_f));
     L.tw = walign16(std::max(cg_end, setup));
-    L.red = walign16(L.tw + (size_t)2 * 16 * (kWBN + 2 * kWMaxB) * sizeof(float2));
-    L.total = walign16(L.red + (size_t)2 * band * sizeof(float));
+    L.total = walign16(L.tw + (size_t)2 * 16 * (kWBN + 2 * kWMaxB) * sizeof(float2));
     return L;
 }
 
@@ -486,14 +488,15 @@ namespace {
 struct DFWCtx {
     HWw w;                  // half-warp areas of the CG grids
     HWw ws;                 // half-warp areas of the 512-point setup transforms
-    const float2* tw_n;     // step twiddles of the camera grid
+    float2* tw_n;           // step twiddles of the camera grid (filled per image)
     float2* tw_x;           // step twiddles of the image's row grid (filled per image)
     float2* tw_y;           // step twiddles of the image's column grid (filled per image)
     float2 *GU, *GQ, *PF, *bq;
     float2 *dv, *sv, *wv, *xv;
     float2* stage;          // stages of the setup column pass (alias the half-warp areas)
-    float* rs;              // two lists of the U rows' sums, n_rs entries each
     int n_rs;
+    // two lists of the U rows' sums, n_rs entries each (at most 8 KB) in the place of tw_n
+    __device__ float* rs(int i) const { return reinterpret_cast<float*>(tw_n) + i * n_rs; }
 };
 
 // plain twiddle table of a 16 G-point grid of the wide solve
@@ -515,6 +518,7 @@ __device__ __forceinline__ int dfw_solve(const DFWCtx& c, const DevPlan& P, cons
     const int *urp = P.d_rowptr + D.urp, *qrp = P.d_rowptr + D.qrp, *prp = P.d_rowptr + D.prp;
     const unsigned* qmask = P.d_qmask + D.qmask_off;
     const WValKnown<CL> pval{sp, ph, P.dP_ap + p_off, P.dP_pup + p_off};
+    make_step_twiddles(c.tw_n, P.tw_n, kWBN);
     make_step_twiddles(c.tw_x, wgrid_table(P, BX), BX);
     make_step_twiddles(c.tw_y, wgrid_table(P, BY), BY);
     __syncthreads();
@@ -540,11 +544,11 @@ __device__ __forceinline__ int dfw_solve(const DFWCtx& c, const DevPlan& P, cons
     wpass_rows_in<BX>(w, c.tw_x, c.GQ, mx, nQ, qrp, P.dQ_x + q_off, WValB{c.bq});
     tile_sync<CL>();
     wpass_cols<BY, CL>(w, c.tw_y, mx, c.GQ, mx, nQ, c.GU, mx, nU, WMidTimesField<BY, false>{c.PF});
-    wpass_rows_out<BX, CL>(w, c.tw_x, c.GU, mx, nU, urp, P.dU_x + u_off, WOutStart{c.sv, c.dv, c.xv}, c.rs);
+    wpass_rows_out<BX, CL>(w, c.tw_x, c.GU, mx, nU, urp, P.dU_x + u_off, WOutStart{c.sv, c.dv, c.xv}, c.rs(0));
     tile_sync<CL>();
     // CGNR; each half-warp updates the vector entries of the U rows it gathered. Every warp
     // forms the scalars itself, from the same sums in the same order.
-    FF gamma = row_total(c.rs, nU);
+    FF gamma = row_total(c.rs(0), nU);
     const CgStop stop(tol, gamma.hi);
     bool conv = !(gamma.hi > 0.f);
     int it = 0;
@@ -555,9 +559,9 @@ __device__ __forceinline__ int dfw_solve(const DFWCtx& c, const DevPlan& P, cons
         wpass_cols<BY, CL>(w, c.tw_y, mx, c.GU, mx, nU, c.GQ, mx, nQ, WMidTimesField<BY, true>{c.PF});
         wpass_rows_mask<BX, CL>(w, c.tw_x, c.GQ, nQ, qmask);
         wpass_cols<BY, CL>(w, c.tw_y, mx, c.GQ, mx, nQ, c.GU, mx, nU, WMidTimesField<BY, false>{c.PF});
-        wpass_rows_out<BX, CL>(w, c.tw_x, c.GU, mx, nU, urp, P.dU_x + u_off, WOutDot{c.wv, c.dv}, c.rs);
+        wpass_rows_out<BX, CL>(w, c.tw_x, c.GU, mx, nU, urp, P.dU_x + u_off, WOutDot{c.wv, c.dv}, c.rs(0));
         tile_sync<CL>();
-        const FF delta = row_total(c.rs, nU);
+        const FF delta = row_total(c.rs(0), nU);
         if (!(delta.hi > 0.f)) break;
         const float af = ff_div(gamma, delta);
         for (int b = w.gh; b < nU; b += w.ghs) {
@@ -572,10 +576,10 @@ __device__ __forceinline__ int dfw_solve(const DFWCtx& c, const DevPlan& P, cons
                 c.sv[e] = sv;
                 g2 += sv.x * sv.x + sv.y * sv.y;
             }
-            wrow_sum<CL>(w, g2, b, c.rs + c.n_rs);
+            wrow_sum<CL>(w, g2, b, c.rs(1));
         }
         tile_sync<CL>();
-        const FF gnew = row_total(c.rs + c.n_rs, nU);
+        const FF gnew = row_total(c.rs(1), nU);
         bf = ff_div(gnew, gamma);
         conv = stop.reached(gnew.hi);
         gamma = gnew;
@@ -609,13 +613,10 @@ k_darkfield_wide(DevPlan P, int n_tiles, const float* __restrict__ I, const floa
     c.wv = c.sv + P.max_N;
     c.xv = c.wv + P.max_N;
     c.stage = reinterpret_cast<float2*>(sbase);
-    float2* tw_n = reinterpret_cast<float2*>(sbase + SL.tw);
-    c.tw_n = tw_n;
-    c.tw_x = tw_n + 2 * 16 * kWBN;
+    c.tw_n = reinterpret_cast<float2*>(sbase + SL.tw);
+    c.tw_x = c.tw_n + 2 * 16 * kWBN;
     c.tw_y = c.tw_x + 2 * 16 * kWMaxB;
-    c.rs = reinterpret_cast<float*>(sbase + SL.red);
     c.n_rs = P.band_u;
-    make_step_twiddles(tw_n, P.tw_n, kWBN);
 
     const int rank = CL ? (int)cta_rank() : 0, K = CL ? (int)cta_count() : 1;
     const int slot = blockIdx.x / K, nslots = gridDim.x / K;      // tile slot = the cluster

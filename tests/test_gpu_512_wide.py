@@ -1,0 +1,38 @@
+"""512-pixel darkfield kernel: plans at the limit of its shared memory."""
+import numpy as np
+import pytest
+
+from helpers import as_complex, rel_l2
+from paper_2407_20469_gb300 import apic, learn, synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+FIELD_TOL = 1e-3               # the workload's bar
+
+
+@pytest.mark.parametrize("ill", [synth.illumination(8, ((0.29, 8, 0.0), (0.376, 8, 22.5))),
+                                 synth.illumination(8, ((0.31, 8, 0.0), (0.392, 8, 22.5))),
+                                 synth.illumination_12_22()])
+def test_most_unknowns_that_fit_a_block(ill):
+    """Images of up to 3933, 3940 and 3954 unknowns: their CG vectors leave no 2 KB of a block's
+    shared memory beside the transforms, and the register kernel still takes them; its field is
+    that of the shared-memory kernels."""
+    plan = apic.Plan.from_illumination(512, ill, max_tiles=1)
+    unknowns = max(int(plan.df_set(i, 0)[1][2]) for i in range(plan.info.n_df))
+    assert 3902 < unknowns <= 3967
+    I = learn.simulate(plan, learn.coefficients(learn.field_table(), np.zeros((1, 2), np.float32)),
+                       np.zeros(1, dtype=bool), 5)
+    assert plan.autotune(1, I)["darkfield_register"] > 0
+    out = []
+    for flags in (0, apic.APIC_LEGACY_KERNELS):
+        plan = apic.Plan.from_illumination(512, ill, max_tiles=1, flags=flags)
+        H = plan.info.out_h
+        f = torch.zeros((1, H, 2 * H), device="cuda")
+        z = torch.zeros((1, 15), device="cuda")
+        st = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+        plan.reconstruct_batch(1, I, f, z, None, st)
+        torch.cuda.synchronize()
+        assert int(st) == 0
+        out.append(as_complex(f)[0])
+    assert rel_l2(out[0], out[1]) < FIELD_TOL
