@@ -28,8 +28,8 @@
 // every block takes the same steps. With K blocks per tile only 1/K as many tiles are
 // in flight, so their band grids stay in L2 instead of going to HBM. Data another
 // block wrote is read with L2-only loads (no stale L1 lines).
-// Transforms, vectors and the sums within a row FP32; the sums across rows as float pairs
-// (about 48 bits).
+// Transforms, vectors and the sums within a row FP32; the sums across rows and the CG's
+// scalars to more than FP64's precision (rowsum.cuh).
 #define APIC_PACKED_ADDS 1
 #include <math.h>
 
@@ -445,8 +445,8 @@ __device__ __noinline__ void wpass_image_rows(HWw w, const float2* tw, const flo
 //                     stage, or the output stage of the image columns
 //   [tw, total)       step twiddles of the camera grid and of the image's row and
 //                     column grids. The camera grid's serve an image's setup alone and are
-//                     made anew for each image; during the CG two lists of the U rows' sums
-//                     take their place. (Beside them the lists took 2 KB, and plans whose CG
+//                     made anew for each image; during the CG its scalars and two lists of the
+//                     U rows' sums take their place. (Beside them the lists took 2 KB, and plans whose CG
 //                     vectors fill the block lost this kernel: 3967 unknowns fit, 3902 did
 //                     then; 8 + 16 images on rings at NA 0.29 and 0.376 have 3933.)
 struct DFWSmem {
@@ -495,8 +495,10 @@ struct DFWCtx {
     float2 *dv, *sv, *wv, *xv;
     float2* stage;          // stages of the setup column pass (alias the half-warp areas)
     int n_rs;
-    // two lists of the U rows' sums, n_rs entries each (at most 8 KB) in the place of tw_n
-    __device__ float* rs(int i) const { return reinterpret_cast<float*>(tw_n) + i * n_rs; }
+    // in the place of tw_n (8 KB) during the CG: its scalars and two lists of the U rows'
+    // sums, n_rs entries each (at most the 320 of the longest grid)
+    __device__ CgScalars* cg() const { return reinterpret_cast<CgScalars*>(tw_n); }
+    __device__ float* rs(int i) const { return reinterpret_cast<float*>(cg() + 1) + i * n_rs; }
 };
 
 // plain twiddle table of a 16 G-point grid of the wide solve
@@ -546,24 +548,19 @@ __device__ __forceinline__ int dfw_solve(const DFWCtx& c, const DevPlan& P, cons
     wpass_cols<BY, CL>(w, c.tw_y, mx, c.GQ, mx, nQ, c.GU, mx, nU, WMidTimesField<BY, false>{c.PF});
     wpass_rows_out<BX, CL>(w, c.tw_x, c.GU, mx, nU, urp, P.dU_x + u_off, WOutStart{c.sv, c.dv, c.xv}, c.rs(0));
     tile_sync<CL>();
-    // CGNR; each half-warp updates the vector entries of the U rows it gathered. Every warp
-    // forms the scalars itself, from the same sums in the same order.
-    FF gamma = row_total(c.rs(0), nU);
-    const CgStop stop(tol, gamma.hi);
-    bool conv = !(gamma.hi > 0.f);
+    // CGNR; each half-warp updates the vector entries of the U rows it gathered
+    bool conv = cg_start(c.cg(), c.rs(0), nU, tol);
     int it = 0;
-    float bf = 0.f;
     for (; it < iters && !conv; ++it) {
-        wpass_rows_in<BX>(w, c.tw_x, c.GU, mx, nU, urp, P.dU_x + u_off, WValNextDir{c.sv, c.dv, bf});
+        wpass_rows_in<BX>(w, c.tw_x, c.GU, mx, nU, urp, P.dU_x + u_off, WValNextDir{c.sv, c.dv, c.cg()->beta});
         tile_sync<CL>();
         wpass_cols<BY, CL>(w, c.tw_y, mx, c.GU, mx, nU, c.GQ, mx, nQ, WMidTimesField<BY, true>{c.PF});
         wpass_rows_mask<BX, CL>(w, c.tw_x, c.GQ, nQ, qmask);
         wpass_cols<BY, CL>(w, c.tw_y, mx, c.GQ, mx, nQ, c.GU, mx, nU, WMidTimesField<BY, false>{c.PF});
         wpass_rows_out<BX, CL>(w, c.tw_x, c.GU, mx, nU, urp, P.dU_x + u_off, WOutDot{c.wv, c.dv}, c.rs(0));
         tile_sync<CL>();
-        const FF delta = row_total(c.rs(0), nU);
-        if (!(delta.hi > 0.f)) break;
-        const float af = ff_div(gamma, delta);
+        if (!cg_alpha(c.cg(), c.rs(0), nU)) break;
+        const float af = c.cg()->alpha;
         for (int b = w.gh; b < nU; b += w.ghs) {
             float g2 = 0.f;
             for (int e = urp[b] + w.t; e < urp[b + 1]; e += 16) {
@@ -579,10 +576,7 @@ __device__ __forceinline__ int dfw_solve(const DFWCtx& c, const DevPlan& P, cons
             wrow_sum<CL>(w, g2, b, c.rs(1));
         }
         tile_sync<CL>();
-        const FF gnew = row_total(c.rs(1), nU);
-        bf = ff_div(gnew, gamma);
-        conv = stop.reached(gnew.hi);
-        gamma = gnew;
+        conv = cg_beta(c.cg(), c.rs(1), nU);
     }
     // corrected unknown spectrum into the tile's spectrum (this block's U rows)
     const int* Upup = P.dU_pup + u_off;

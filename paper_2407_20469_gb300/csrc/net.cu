@@ -30,7 +30,6 @@
 #include "internal.cuh"
 #include "netconv.cuh"
 #include "regfft.cuh"
-#include "rowsum.cuh"
 #include "t4grid.cuh"
 
 namespace apic {
@@ -94,6 +93,15 @@ struct FeatCfg {
     static constexpr int threads = BN <= 16 ? 256 : 512, blocks = BN == 16 ? 3 : BN == 8 ? 2 : 1;
 };
 
+// An unevaluated sum hi + lo of floats; Knuth's two-sum makes it exact for two floats.
+struct FF {
+    float hi, lo;
+};
+__device__ __forceinline__ FF ff_two_sum(float a, float b) {
+    const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z))};
+}
+
 template <int BN>
 __global__ void __launch_bounds__(FeatCfg<BN>::threads, FeatCfg<BN>::blocks)
 k_features(DevPlan P, int n_tiles, const float* __restrict__ I, float* __restrict__ feat, float2* __restrict__ scratch) {
@@ -112,7 +120,7 @@ k_features(DevPlan P, int n_tiles, const float* __restrict__ I, float* __restric
     for (int prob = blockIdx.x; prob < nprob; prob += gridDim.x) {
         const int tile = prob / kIn, i = prob - tile * kIn;
         const float* img = I + ((size_t)tile * P.n_img + i) * n * n;
-        // the image's sum on the way: per thread as a float pair (rowsum.cuh; an FP64 add per
+        // the image's sum on the way: per thread as a float pair (an FP64 add per
         // pixel kept the FP64 pipe busy for a quarter of the kernel's time), across threads in
         // FP64
         FF sum = {0.f, 0.f};

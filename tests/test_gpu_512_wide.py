@@ -36,3 +36,42 @@ def test_most_unknowns_that_fit_a_block(ill):
         assert int(st) == 0
         out.append(as_complex(f)[0])
     assert rel_l2(out[0], out[1]) < FIELD_TOL
+
+
+def _stitched(tile, ill, n):
+    """Plan, intensities, coefficients and stitched spectrum: the darkfield stage's inputs."""
+    plan = apic.Plan.from_illumination(tile, ill, max_tiles=n)
+    zern = learn.coefficients(learn.field_table(), np.zeros((n, 2), np.float32))
+    I = learn.simulate(plan, zern, np.zeros(n, dtype=bool), 5)
+    info = plan.info
+    x = torch.empty((n, info.n_bf, info.n_pupil, 2), device="cuda")
+    z = torch.empty((n, 15), device="cuda")
+    spec = torch.empty((n, info.n_aperture, 2), device="cuda")
+    plan.kk_spectra(n, I, x)
+    plan.aberration(n, x, z)
+    plan.stitch(n, x, z, spec)
+    return plan, I, z, spec
+
+
+def test_intensity_scale():
+    """Intensities times 2^t with a spectrum times 2^(t/2): every FP32 operation of the solve then
+    scales by a power of two, so the result does too, bit for bit, while no product or sum of a
+    row leaves FP32's range (the sums over all rows do before: at 2^41). Beyond, a tile's solve
+    may end early, but never unflagged."""
+    plan, I, z, spec = _stitched(512, synth.illumination_8_24(), 1)
+
+    def solve(t):
+        s = spec * 2.0 ** (t % 2 / 2) * 2.0 ** (t // 2)
+        st = torch.zeros(1, dtype=torch.int32, device="cuda")
+        plan.darkfield(1, I * 2.0 ** t, z, s, st)
+        torch.cuda.synchronize()
+        return s, int(st)
+
+    base = [solve(t) for t in (0, 1)]
+    assert all(st == 0 for _, st in base)
+    for t in (-10, 2, 20, 35, 38, 40, 41):
+        s, st = solve(t)
+        assert st == 0 and torch.equal(s, base[t % 2][0] * 2.0 ** (t // 2)), t
+    for t in range(42, 75):
+        s, st = solve(t)
+        assert st == apic.APIC_TILE_NOTCONV or torch.equal(s, base[t % 2][0] * 2.0 ** (t // 2)), t
