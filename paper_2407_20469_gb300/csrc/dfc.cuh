@@ -707,8 +707,10 @@ template <int BN, int B>
 __global__ void __launch_bounds__(kClThreads, 1)
 k_darkfield_cluster(DevPlan P, ClSmem L, int n_tiles, const float* __restrict__ I, const float* __restrict__ phi,
                     float2* __restrict__ spec, char* __restrict__ scratch, size_t per_slot, int iters, float tol,
-                    int32_t* __restrict__ status, unsigned long long* __restrict__ counters) {
+                    int32_t* __restrict__ status, unsigned long long* __restrict__ counters, DfTiles T) {
     constexpr int n = 16 * BN;
+    n_tiles = T.count(n_tiles);
+    if (n_tiles <= 0) return;
     extern __shared__ float4 smem4[];
     __shared__ uint32_t tmem_base;
     ClCtx c;
@@ -748,7 +750,8 @@ k_darkfield_cluster(DevPlan P, ClSmem L, int n_tiles, const float* __restrict__ 
     c.ws.hs = reinterpret_cast<float2*>(c.smem) + c.ws.hw * hw_single_size(BN > B ? BN : B);
     cl_sync();           // every block of the cluster runs before any stores into another's shared memory
 
-    for (int tile = slot; tile < n_tiles; tile += nslots) {
+    for (int i = slot; i < n_tiles; i += nslots) {
+        const int tile = T.tile(i);
         if (status && (status[tile] & (APIC_TILE_BACKGROUND | APIC_TILE_BADINPUT))) continue;
         const float* ph = phi + (size_t)tile * P.npup;
         float2* sp = spec + (size_t)tile * P.nap;
@@ -778,7 +781,7 @@ k_darkfield_cluster(DevPlan P, ClSmem L, int n_tiles, const float* __restrict__ 
 }  // namespace
 
 using ClKernel = void (*)(DevPlan, ClSmem, int, const float*, const float*, float2*, char*, size_t, int, float,
-                          int32_t*, unsigned long long*);
+                          int32_t*, unsigned long long*, DfTiles);
 
 // The kernel of 256-pixel tiles for a register grid of 16 B points (NULL: none); a translation unit of its own.
 ClKernel cl_kernel_256(int B);

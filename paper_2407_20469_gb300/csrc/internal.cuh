@@ -144,6 +144,18 @@ cudaError_t launch_sim(const DevPlan& P, const Launch& L, int n_tiles, const flo
 
 size_t df_scratch_bytes(const DevPlan& P);
 
+// Tiles of one of a batch's darkfield launches: all of them in order (list NULL), or entries
+// first, first + 1, ... of a list of the tiles to solve: list[0] their number, then the tiles.
+struct DfTiles {
+    const int* list = nullptr;
+    int first = 0;
+
+    __device__ int count(int n_tiles) const { return list ? min(n_tiles, list[0] - first) : n_tiles; }
+    __device__ int tile(int i) const { return list ? list[1 + first + i] : i; }
+};
+// The tiles of a batch that are not skipped, into list (n_tiles + 1 entries)
+cudaError_t launch_list_tiles(int n_tiles, const int32_t* status, int* list, cudaStream_t st);
+
 // register-FFT darkfield kernel (m = 16 B, n = 16 BN)
 size_t dfr_smem_bytes(int B, int BN, int band_u, int band_q, int max_N);
 size_t dfr_scratch_bytes(const DevPlan& P);
@@ -153,7 +165,7 @@ int configure_dfr(int B, int BN, size_t smem);
 cudaError_t launch_darkfield_reg(const DevPlan& P, int grid, size_t smem, int n_tiles, const float* I,
                                  const float* phi, float2* spec, void* scratch, size_t per_block, int iters,
                                  float tol, int32_t* status, unsigned long long* counters, int* work,
-                                 cudaStream_t st);
+                                 cudaStream_t st, DfTiles tiles = {});
 
 // cluster darkfield kernel of 128- and 256-pixel tiles (dfc.cuh): K blocks per tile, the band
 // grids in their shared memory. configure_dfc returns the clusters that run at once for the
@@ -163,7 +175,7 @@ int configure_dfc(const DevPlan& P, int K);
 size_t dfc_scratch_bytes(const DevPlan& P);
 cudaError_t launch_darkfield_cluster(const DevPlan& P, int K, int slots, int n_tiles, const float* I, const float* phi,
                                      float2* spec, void* scratch, int iters, float tol, int32_t* status,
-                                     unsigned long long* counters, cudaStream_t st);
+                                     unsigned long long* counters, cudaStream_t st, DfTiles tiles = {});
 
 // wide darkfield kernel of 512-pixel tiles (kernels_dfw.cu)
 size_t dfw_smem_bytes(int max_N, int band);   // band: max of the U, P and Q row bands
@@ -173,7 +185,7 @@ int configure_dfw(size_t smem, int K);
 cudaError_t launch_darkfield_wide(const DevPlan& P, int K, int grid, size_t smem, int n_tiles, const float* I,
                                   const float* phi, float2* spec, void* scratch, size_t per_block, int iters,
                                   float tol, int32_t* status, unsigned long long* counters, int* work,
-                                  cudaStream_t st);
+                                  cudaStream_t st, DfTiles tiles = {});
 
 // Network features (net.cu): feat [n_tiles][64][64][8] from the first 8 images
 // of each stack, on at most `grid` SMs; `scratch` holds h * h complex values for each.

@@ -43,14 +43,14 @@ int configure_dfc(const DevPlan& P, int K) {
 
 cudaError_t launch_darkfield_cluster(const DevPlan& P, int K, int slots, int n_tiles, const float* I, const float* phi,
                                      float2* spec, void* scratch, int iters, float tol, int32_t* status,
-                                     unsigned long long* counters, cudaStream_t st) {
+                                     unsigned long long* counters, cudaStream_t st, DfTiles tiles) {
     ClKernel f = cl_kernel(P);
     slots = std::min(slots, n_tiles);
     if (!f) return cudaErrorInvalidValue;
     if (slots < 1) return cudaErrorInvalidConfiguration;
     const ClSmem L = cl_layout(P, K);
     return cluster_launch(f, K, slots, kClThreads, cl_smem_bytes(L), st, P, L, n_tiles, I, phi, spec, (char*)scratch,
-                          dfc_scratch_bytes(P), iters, tol, status, counters);
+                          dfc_scratch_bytes(P), iters, tol, status, counters, tiles);
 }
 
 }  // namespace apic

@@ -794,8 +794,11 @@ template <int B, int BN>
 __global__ void __launch_bounds__(kDFThreads, 1)
 k_darkfield_reg(DevPlan P, int n_tiles, const float* __restrict__ I, const float* __restrict__ phi,
                 float2* __restrict__ spec, char* __restrict__ scratch, size_t per_block, int iters, float tol,
-                int32_t* __restrict__ status, unsigned long long* __restrict__ counters, int* __restrict__ work) {
+                int32_t* __restrict__ status, unsigned long long* __restrict__ counters, int* __restrict__ work,
+                DfTiles T) {
     constexpr int m = 16 * B, n = 16 * BN;
+    n_tiles = T.count(n_tiles);
+    if (n_tiles <= 0) return;
     constexpr int HWM = hw_area_m(B), HWN = HWSize<BN>::value;
     extern __shared__ float4 smem4[];
     char* sbase = reinterpret_cast<char*>(smem4);
@@ -862,7 +865,8 @@ k_darkfield_reg(DevPlan P, int n_tiles, const float* __restrict__ I, const float
         __syncthreads();
         return s_next;
     };
-    for (int tile = take(-1); tile < n_tiles; tile = take(tile)) {
+    for (int i = take(-1); i < n_tiles; i = take(i)) {
+        const int tile = T.tile(i);
         if (status && (status[tile] & (APIC_TILE_BACKGROUND | APIC_TILE_BADINPUT))) continue;
         const float* ph = phi + (size_t)tile * P.npup;
         float2* sp = spec + (size_t)tile * P.nap;
@@ -909,7 +913,7 @@ k_darkfield_reg(DevPlan P, int n_tiles, const float* __restrict__ I, const float
 }
 
 using DFRKernel = void (*)(DevPlan, int, const float*, const float*, float2*, char*, size_t, int, float, int32_t*,
-                           unsigned long long*, int*);
+                           unsigned long long*, int*, DfTiles);
 
 DFRKernel dfr_kernel(int B, int BN) {
     if (B == 4 && BN == 4) return k_darkfield_reg<4, 4>;
@@ -932,7 +936,8 @@ int configure_dfr(int B, int BN, size_t smem) {
 
 cudaError_t launch_darkfield_reg(const DevPlan& P, int grid, size_t smem, int n_tiles, const float* I,
                                  const float* phi, float2* spec, void* scratch, size_t per_block, int iters,
-                                 float tol, int32_t* status, unsigned long long* counters, int* work, cudaStream_t st) {
+                                 float tol, int32_t* status, unsigned long long* counters, int* work, cudaStream_t st,
+                                 DfTiles tiles) {
     DFRKernel f = dfr_kernel(P.mr / 16, P.h / 16);
     if (!f) return cudaErrorInvalidValue;
     if (work) {
@@ -940,7 +945,7 @@ cudaError_t launch_darkfield_reg(const DevPlan& P, int grid, size_t smem, int n_
         if (e != cudaSuccess) return e;
     }
     f<<<min(grid, n_tiles), kDFThreads, smem, st>>>(P, n_tiles, I, phi, spec, (char*)scratch, per_block, iters, tol,
-                                                  status, counters, work);
+                                                  status, counters, work, tiles);
     return cudaGetLastError();
 }
 

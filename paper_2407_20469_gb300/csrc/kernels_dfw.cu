@@ -596,8 +596,11 @@ template <bool CL>
 __global__ void __launch_bounds__(kWThreads, 1)
 k_darkfield_wide(DevPlan P, int n_tiles, const float* __restrict__ I, const float* __restrict__ phi,
                  float2* __restrict__ spec, char* __restrict__ scratch, size_t per_block, int iters, float tol,
-                 int32_t* __restrict__ status, unsigned long long* __restrict__ counters, int* __restrict__ work) {
+                 int32_t* __restrict__ status, unsigned long long* __restrict__ counters, int* __restrict__ work,
+                 DfTiles T) {
     constexpr int n = 16 * kWBN;
+    n_tiles = T.count(n_tiles);
+    if (n_tiles <= 0) return;
     extern __shared__ float4 smem4[];
     char* sbase = reinterpret_cast<char*>(smem4);
     const DFWSmem SL = dfw_smem_layout(P.max_N, max(P.band_q, max(P.band_p, P.band_u)));
@@ -640,7 +643,8 @@ k_darkfield_wide(DevPlan P, int n_tiles, const float* __restrict__ I, const floa
         __syncthreads();
         return s_next;
     };
-    for (int tile = take(-1); tile < n_tiles; tile = take(tile)) {
+    for (int i = take(-1); i < n_tiles; i = take(i)) {
+        const int tile = T.tile(i);
         if (status && (status[tile] & (APIC_TILE_BACKGROUND | APIC_TILE_BADINPUT))) continue;
         const float* ph = phi + (size_t)tile * P.npup;
         float2* sp = spec + (size_t)tile * P.nap;
@@ -672,7 +676,7 @@ k_darkfield_wide(DevPlan P, int n_tiles, const float* __restrict__ I, const floa
 }  // namespace
 
 using DFWKernel = void (*)(DevPlan, int, const float*, const float*, float2*, char*, size_t, int, float, int32_t*,
-                           unsigned long long*, int*);
+                           unsigned long long*, int*, DfTiles);
 
 static DFWKernel dfw_kernel(int K) {
     return K == 1 ? k_darkfield_wide<false> : K >= 2 && K <= kMaxCluster ? k_darkfield_wide<true> : nullptr;
@@ -685,7 +689,7 @@ int configure_dfw(size_t smem, int K) { return cluster_slots((const void*)dfw_ke
 cudaError_t launch_darkfield_wide(const DevPlan& P, int K, int grid, size_t smem, int n_tiles, const float* I,
                                   const float* phi, float2* spec, void* scratch, size_t per_block, int iters,
                                   float tol, int32_t* status, unsigned long long* counters, int* work,
-                                  cudaStream_t st) {
+                                  cudaStream_t st, DfTiles tiles) {
     DFWKernel f = dfw_kernel(K);
     if (!f || P.h != 16 * kWBN || P.w != P.h) return cudaErrorInvalidValue;
     const int slots = min(grid, n_tiles);
@@ -695,7 +699,7 @@ cudaError_t launch_darkfield_wide(const DevPlan& P, int K, int grid, size_t smem
         if (e != cudaSuccess) return e;
     }
     return cluster_launch(f, K, slots, kWThreads, smem, st, P, n_tiles, I, phi, spec, (char*)scratch, per_block, iters,
-                          tol, status, counters, K == 1 ? work : (int*)nullptr);
+                          tol, status, counters, K == 1 ? work : (int*)nullptr, tiles);
 }
 
 }  // namespace apic

@@ -94,6 +94,36 @@ __device__ __forceinline__ bool skip_tile(const int32_t* status, int tile) {
     return status && (status[tile] & (APIC_TILE_BACKGROUND | APIC_TILE_BADINPUT));
 }
 
+// The tiles that are not skipped, in order: list[0] their number, list[1 ..] the tiles. One
+// block, 1024 tiles at a time.
+__global__ void __launch_bounds__(1024) k_list_tiles(int n_tiles, const int32_t* __restrict__ status,
+                                                     int* __restrict__ list) {
+    __shared__ int warps[32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int found = 0;
+    for (int t0 = 0; t0 < n_tiles; t0 += 1024) {
+        const int tile = t0 + threadIdx.x;
+        const bool on = tile < n_tiles && !skip_tile(status, tile);
+        const unsigned mask = __ballot_sync(0xffffffffu, on);
+        if (lane == 0) warps[warp] = __popc(mask);
+        __syncthreads();
+        int before = 0, all = 0;
+        for (int w = 0; w < 32; ++w) {
+            before += w < warp ? warps[w] : 0;
+            all += warps[w];
+        }
+        if (on) list[1 + found + before + __popc(mask & ((1u << lane) - 1))] = tile;
+        found += all;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) list[0] = found;
+}
+
+cudaError_t launch_list_tiles(int n_tiles, const int32_t* status, int* list, cudaStream_t st) {
+    k_list_tiles<<<1, 1024, 0, st>>>(n_tiles, status, list);
+    return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------- Kramers-Kronig
 // One block per (tile, NA-matching image) problem, persistent over problems.
 // Scratch: an n x n complex grid per block.
