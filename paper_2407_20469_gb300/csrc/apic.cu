@@ -100,7 +100,6 @@ struct apic_plan {
     int df_slots[kMaxCluster + 1] = {};   // register darkfield kernels: tile slots with K blocks per tile
     int df_slots_alloc = 0;      // tile slots of each half of the darkfield scratch
     int kk_slots[kMaxCluster + 1] = {};   // Kramers-Kronig problems at once with K (a power of 2) blocks each
-    bool df_rounds = true;       // small batches in rounds of several blocks per tile (off while autotuning)
     // host-buffer pipeline (apic_reconstruct_host), created on first use
     struct HostIO {
         bool ready = false;
@@ -663,7 +662,7 @@ DfRounds df_schedule(const apic_plan* p, int n) {
     return r;
 }
 
-bool df_may_cluster(const apic_plan* p) { return p->use_reg && p->df_rounds && p->df_cluster == 1; }
+bool df_may_cluster(const apic_plan* p) { return p->use_reg && p->df_cluster == 1; }
 
 // Rounds behind full waves that take more than this many round times are not worth a
 // launch of their own: in one launch blocks that come free early go on to the last tiles.
@@ -1785,7 +1784,6 @@ apic_status apic_plan_autotune(apic_plan* plan, int n_tiles, const float* I, dou
     // stitched spectrum, so repeated runs see the same system
     const bool had_reg = plan->use_reg;
     const bool wide = D.mr == 512;
-    plan->df_rounds = false;             // the variants themselves, not a small batch's rounds
     const int had_k = plan->df_cluster, had_grid = plan->grid_dfr;
     void* scratch[2] = {nullptr, nullptr};
     size_t per_block[2] = {wide ? dfw_scratch_bytes(D) : dfr_scratch_bytes(D), df_scratch_bytes(D)};
@@ -1804,13 +1802,16 @@ apic_status apic_plan_autotune(apic_plan* plan, int n_tiles, const float* I, dou
         plan->df_scratch = scratch[v];
         plan->df_per_block = per_block[v];
         plan->df_slots_alloc = slots_alloc[v];
-        if (v == 0 && wide) {      // the wide kernel at each cluster size: blocks per tile 1, 2, 4
+        // the wide kernel at each cluster size: blocks per tile 1 (with the rounds of launch_df, as
+        // the plan runs it), 2 and 4. A fixed 2 or 4 ends the rounds, for every later batch; a
+        // sample below a full wave, which the rounds serve best, cannot speak for that.
+        if (v == 0 && wide) {
             for (int i = 0; i < 3 && err == cudaSuccess; ++i) {
                 if (plan->df_slots[1 << i] <= 0) continue;
                 plan->df_cluster = 1 << i;
                 plan->grid_dfr = plan->df_slots[1 << i];
                 err = timed([&] { return launch_df(plan, n_tiles, I, plan->spec, stt, st); }, ms[4 + i]);
-                if (err == cudaSuccess && (ms[2] < 0 || ms[4 + i] < ms[2])) {
+                if (err == cudaSuccess && (ms[2] < 0 || (ms[4 + i] < ms[2] && n_tiles >= plan->df_slots[1]))) {
                     ms[2] = ms[4 + i];
                     best_k = plan->df_cluster;
                     best_grid = plan->grid_dfr;
@@ -1842,7 +1843,6 @@ apic_status apic_plan_autotune(apic_plan* plan, int n_tiles, const float* I, dou
         plan->df_cluster = had_k;
         plan->grid_dfr = had_grid;
     }
-    plan->df_rounds = true;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaStreamDestroy(st);

@@ -1,4 +1,7 @@
-"""512-pixel darkfield kernel: plans at the limit of its shared memory."""
+"""512-pixel darkfield kernel: plans at the limit of its shared memory, intensities up to the limit of
+FP32, autotuning on a few tiles."""
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -75,3 +78,23 @@ def test_intensity_scale():
     for t in range(42, 75):
         s, st = solve(t)
         assert st == apic.APIC_TILE_NOTCONV or torch.equal(s, base[t % 2][0] * 2.0 ** (t // 2)), t
+
+
+def _wave(plan):
+    info = apic.apic_plan_info()
+    assert apic.load().apic_plan_query(plan.handle, C.byref(info)) == apic.APIC_OK
+    return info.df_wave
+
+
+def test_autotune_on_a_few_tiles_keeps_the_rounds():
+    """A sample below a wave leaves the plan at one block per tile by default, so that batches
+    below a wave still go in rounds; results and waves are those of an untuned plan."""
+    plan, I, z, spec = _stitched(512, synth.illumination_8_24(), 4)
+    wave = _wave(plan)
+    a, b = spec.clone(), spec.clone()
+    plan.darkfield(4, I, z, a)
+    ms = plan.autotune(4, I)
+    assert all(ms[k] > 0 for k in ms)
+    assert _wave(plan) == wave
+    plan.darkfield(4, I, z, b)
+    assert torch.equal(a, b)
