@@ -425,7 +425,7 @@ apic_status configure(apic_plan* plan) {
     plan->kkr_ok = plan->dfr_ok = false;
     if (D.h == D.w && (D.h == 64 || D.h == 128 || D.h == 256 || D.h == 512)) {
         const size_t smem = kkr_smem_bytes(D.h / 16);
-        for (int K = 1; K <= kMaxCluster; K *= 2) {
+        for (int K = 1; K <= 8; K *= 2) {
             plan->kk_slots[K] = configure_kkr(D.h / 16, smem, K);
             cudaGetLastError();
         }
@@ -529,13 +529,14 @@ apic_status alloc_workspace(apic_plan* p) {
 // results do not depend on K):
 //   512 px: 0.39 with one block, 0.22 with 2, 0.13 with 4, 0.074 with 8 (16: no faster)
 //   256 px: 0.107, 0.068, 0.044, 0.034;   128 px: 0.046, 0.036, 0.027, 0.027
-// Two blocks at 512 pixels also keep half as many grids in flight (152 MB): 96 tiles
-// 2.50 -> 2.43 ms, 25 tiles 0.83 -> 0.67.
+// 64-pixel tiles stay with one block. At 512 pixels 25 tiles take 0.67 ms by this rule and 0.84
+// with one block each, 96 tiles (one block) 2.51. Two blocks would take 2.44 there, with half
+// as many grids, 152 MB, in flight beside the L2; the rule counts rounds only.
 cudaError_t launch_kk_any(apic_plan* p, int blocks, int n_tiles, const float* I, float2* xdisc, float2* scratch,
                           const int32_t* status, cudaStream_t st, int grids = 0) {
     if (p->use_kkr) {
-        static const double t[4][4] = {{1, 9, 9, 9}, {1, 0.78, 0.60, 0.60}, {1, 0.64, 0.42, 0.33}, {1, 0.57, 0.34, 0.20}};
-        const double* tk = t[p->dev.h == 512 ? 3 : p->dev.h == 256 ? 2 : p->dev.h == 128 ? 1 : 0];
+        static const double t[3][4] = {{1, 0.78, 0.60, 0.60}, {1, 0.64, 0.42, 0.33}, {1, 0.57, 0.34, 0.20}};
+        const double* tk = t[p->dev.h == 512 ? 2 : p->dev.h == 256 ? 1 : 0];
         const int most = blocks > 0 ? std::min(blocks, p->grid_kkr) : p->grid_kkr, nprob = n_tiles * p->dev.n_bf;
         int K = 1, slots = 0;
         double best = 1e30;

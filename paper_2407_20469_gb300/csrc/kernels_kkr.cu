@@ -190,7 +190,7 @@ using KKRKernel = void (*)(DevPlan, int, const float*, float2*, float2*, const i
 
 static KKRKernel kkr_kernel(int BN, int K) {
     switch (BN) {
-        case 4: return K > 1 ? k_kk_reg<4, true> : k_kk_reg<4, false>;
+        case 4: return K > 1 ? nullptr : k_kk_reg<4, false>;
         case 8: return K > 1 ? k_kk_reg<8, true> : k_kk_reg<8, false>;
         case 16: return K > 1 ? k_kk_reg<16, true> : k_kk_reg<16, false>;
         case 32: return K > 1 ? k_kk_reg<32, true> : k_kk_reg<32, false>;
