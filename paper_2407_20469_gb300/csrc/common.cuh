@@ -144,6 +144,8 @@ __device__ __forceinline__ double block_sum2f_ratio(float v, double num, double*
     return total;
 }
 
+}  // inline namespace
+
 // Raises (never lowers) a kernel's dynamic shared-memory limit. The limit is
 // process-wide per function, so plans of different sizes that share a kernel
 // must not shrink it under one another.
@@ -155,5 +157,4 @@ inline cudaError_t raise_smem_limit(const void* f, size_t smem) {
     return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
-}  // inline namespace
 }  // namespace apic
