@@ -394,12 +394,35 @@ apic_status upload(apic_plan* plan) {
     return APIC_OK;
 }
 
+// Blocks per tile K that a round of a darkfield batch may take, and the time t of such a
+// round of as many tiles as run at once (a cluster's blocks share a GPC, so fewer than
+// SMs / K), in times of a round of one block per tile. Measured on a GB300, in milliseconds:
+//   128 px, 8 + 16 images: 5.5 (151 tiles, K = 1), 4.2 (46, 3), 3.3 (28, 5), 3.2 (15, 8)
+//   256 px, 8 + 16: 15.6 (151, 1), 8.4 (46, 3), 6.7 (36, 4), 6.2 (23, 6), 5.0 (15, 8)
+//   512 px, 8 + 24: 69 (151, 1), 40 (76, 2), 29 (46, 3), 25.9 (36, 4), 21.6 (28, 5),
+//   20.3 (23, 6), 18.5 (15, 8), 15.1 (13, 10); K = 16 is no faster than 10 on one tile
+// 64-pixel tiles stay with one block (2.4 ms; clusters were slower).
+struct DfRoundTime {
+    int K;
+    double t;
+};
+
+const DfRoundTime* df_round_times(int h, int& n) {
+    static const DfRoundTime t128[] = {{3, 0.77}, {5, 0.61}, {8, 0.59}};
+    static const DfRoundTime t256[] = {{3, 0.54}, {4, 0.43}, {6, 0.40}, {8, 0.32}};
+    static const DfRoundTime t512[] = {{2, 0.58}, {3, 0.42}, {4, 0.37}, {5, 0.31}, {6, 0.29}, {8, 0.27}, {10, 0.22}};
+    n = h == 128 ? 3 : h == 256 ? 4 : h == 512 ? 7 : 0;
+    return h == 128 ? t128 : h == 256 ? t256 : t512;
+}
+
 // Clusters of K blocks that the cluster kernel of tiles up to 256 pixels runs at once, for the
 // plan's current tables.
 void configure_clusters(apic_plan* plan) {
     if (!plan->dfr_ok || plan->dev.mr == 512) return;
-    for (int K = 2; K <= kMaxCluster; ++K) {
-        plan->df_slots[K] = configure_dfc(plan->dev, K);
+    int n = 0;
+    const DfRoundTime* t = df_round_times(plan->dev.h, n);
+    for (int i = 0; i < n; ++i) {
+        plan->df_slots[t[i].K] = configure_dfc(plan->dev, t[i].K);
         cudaGetLastError();
     }
 }
@@ -445,13 +468,10 @@ apic_status configure(apic_plan* plan) {
             // blocks per tile: 1 by default, the most tiles per second from a full wave on
             // (launch_df takes more for smaller batches; for 512-pixel tiles the
             // autotuner times 1, 2 and 4 and can settle on another default)
-            if (wide)
-                for (int K = 1; K <= kMaxCluster; ++K) {
-                    plan->df_slots[K] = configure_dfw(smem, K);
-                    cudaGetLastError();
-                }
-            else
-                plan->df_slots[1] = sms * configure_dfr(D.mr / 16, D.h / 16, smem);
+            plan->df_slots[1] = wide ? configure_dfw(smem, 1) : sms * configure_dfr(D.mr / 16, D.h / 16, smem);
+            int n = 0;
+            const DfRoundTime* t = df_round_times(D.h, n);
+            for (int i = 0; wide && i < n; ++i) plan->df_slots[t[i].K] = configure_dfw(smem, t[i].K);
             const int pick = plan->df_slots[1] > 0 || !wide ? 1 : 2;
             if (plan->df_slots[pick] > 0) {
                 plan->dfr_ok = true;
@@ -584,15 +604,7 @@ cudaError_t launch_df_on(apic_plan* p, int n_tiles, const float* I, const float*
                             status, p->d_counters, st);
 }
 
-// Ways to solve a round of tiles: K blocks per tile, at most `cap` tiles at once, in `t`
-// times the time of a round of one block per tile. Measured on a GB300, the darkfield
-// stage of as many tiles as run at once (a cluster's blocks share a GPC, so fewer than
-// SMs / K), in milliseconds:
-//   128 px, 8 + 16 images: 5.5 (151 tiles, K = 1), 4.2 (46, 3), 3.3 (28, 5), 3.2 (15, 8)
-//   256 px, 8 + 16: 15.6 (151, 1), 8.4 (46, 3), 6.7 (36, 4), 6.2 (23, 6), 5.0 (15, 8)
-//   512 px, 8 + 24: 69 (151, 1), 40 (76, 2), 29 (46, 3), 25.9 (36, 4), 21.6 (28, 5),
-//   20.3 (23, 6), 18.5 (15, 8), 15.1 (13, 10); K = 16 is no faster than 10 on one tile
-// 64-pixel tiles stay with one block (2.4 ms; clusters were slower).
+// Ways to solve a round of tiles: K blocks per tile, at most `cap` tiles at once, in time t.
 struct DfOption {
     int K, cap;
     double t;
@@ -605,24 +617,15 @@ struct DfOptions {
 };
 
 DfOptions df_options(const apic_plan* p) {
-    static const double t128[][2] = {{3, 0.77}, {5, 0.61}, {8, 0.59}};
-    static const double t256[][2] = {{3, 0.54}, {4, 0.43}, {6, 0.40}, {8, 0.32}};
-    static const double t512[][2] = {{2, 0.58}, {3, 0.42}, {4, 0.37}, {5, 0.31}, {6, 0.29}, {8, 0.27}, {10, 0.22}};
     DfOptions r;
     r.o[r.n++] = {1, p->grid_dfr, 1.0};
-    auto add = [&](const double (*t)[2], int n) {
-        for (int i = 0; i < n; ++i) {
-            // clusters that run at once, and that the scratch of one wave holds
-            const int K = (int)t[i][0];
-            const size_t each = p->dev.mr == 512 ? p->df_per_block : dfc_scratch_bytes(p->dev);
-            const int cap = (int)std::min<size_t>(p->df_slots[K], p->df_slots_alloc * p->df_per_block / each);
-            if (cap > 0) r.o[r.n++] = {K, cap, t[i][1]};
-        }
-    };
-    switch (p->dev.h) {
-        case 128: add(t128, 3); break;
-        case 256: add(t256, 4); break;
-        case 512: add(t512, 7); break;
+    int n = 0;
+    const DfRoundTime* t = df_round_times(p->dev.h, n);
+    for (int i = 0; i < n; ++i) {
+        // clusters that run at once, and that the scratch of one wave holds
+        const size_t each = p->dev.mr == 512 ? p->df_per_block : dfc_scratch_bytes(p->dev);
+        const int cap = (int)std::min<size_t>(p->df_slots[t[i].K], p->df_slots_alloc * p->df_per_block / each);
+        if (cap > 0) r.o[r.n++] = {t[i].K, cap, t[i].t};
     }
     return r;
 }

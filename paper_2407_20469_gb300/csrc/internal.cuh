@@ -170,7 +170,7 @@ cudaError_t launch_darkfield_reg(const DevPlan& P, int grid, size_t smem, int n_
 // cluster darkfield kernel of 128- and 256-pixel tiles (dfc.cuh): K blocks per tile, the band
 // grids in their shared memory. configure_dfc returns the clusters that run at once for the
 // plan's current tables (0: not available); scratch holds dfc_scratch_bytes per cluster.
-constexpr int kMaxCluster = 16;
+constexpr int kMaxCluster = 10;               // blocks per tile or problem, of any kernel
 int configure_dfc(const DevPlan& P, int K);
 size_t dfc_scratch_bytes(const DevPlan& P);
 cudaError_t launch_darkfield_cluster(const DevPlan& P, int K, int slots, int n_tiles, const float* I, const float* phi,

@@ -302,9 +302,6 @@ cudaError_t gemm(int M, int N, int K, int splits, LA la, LB lb, EP ep, cudaStrea
 }
 
 // ---- operand loaders (A(m, k) or B(k, n), returning float)
-__device__ __forceinline__ float to_f(float v) { return v; }
-__device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
-
 struct WT {                 // B(k, n) = W[n][k]; rows padded to multiples of 8
     const __nv_bfloat16* w;
     int ld;
