@@ -210,15 +210,16 @@ apic_status apic_plan_set_df_grid(apic_plan* plan, int index, int mx, int my);
  * aberration solve (Eq. 8-10), correction and stitching, darkfield extension
  * (Eq. 11-13), inverse transform. The global phase of the field is the
  * phase gauge of Eq. 5 (mean phase of the recovered fields set to zero).
- * Batches above max_tiles are processed in chunks. When a chunk is not a
- * whole number of darkfield waves (one tile per block) and its last partial
- * wave holds at most half a wave, that wave's darkfield solves run first, on
- * a second stream the plan owns, forked from and joined back to `stream`
- * (stream capture follows the fork), while the other tiles' earlier stages
- * run on the remaining SMs; a larger partial wave simply ends the darkfield
- * stage. Tiles beyond the last full wave that are not split off, and batches
- * below one wave, are solved by clusters of several thread blocks per tile.
- * Results are identical in every order and with any number of blocks.
+ * Batches above max_tiles are processed in chunks. The darkfield solves of a
+ * chunk go in full waves (one tile per block) and, for the tiles beyond the
+ * last full wave and for chunks below one, in rounds of several thread blocks
+ * per tile (tiles of 128, 256 and 512 pixels) where that is faster. A last
+ * partial wave of at most half a wave may instead run first, one block per
+ * tile, on a second stream the plan owns, forked from and joined back to
+ * `stream` (stream capture follows the fork), while the other tiles' earlier
+ * stages run on the remaining SMs: where hiding those stages saves more than
+ * the rounds do, that is in chunks of many waves. Results are identical in
+ * every order and with any number of blocks.
  */
 apic_status apic_reconstruct_batch(apic_plan* plan, int n_tiles, const float* d_intensity,
                                    float* d_field, float* d_zernike, float* d_pupil,
@@ -343,9 +344,11 @@ apic_status apic_stitch(apic_plan* plan, int n_tiles, const float* d_xdisc,
 
 /*
  * Darkfield extension (Eq. 11-13), darkfield images in plan order, each solved
- * by CGLS on C U = b with FFT correlations (FP32 transforms, FP64 scalars -
- * float pairs at 512 pixels - and solution accumulation). Updates d_spec in place; ORs APIC_TILE_NOTCONV into
- * d_tile_status (may be NULL) where a solve ended above its tolerance.
+ * by CGLS on C U = b with FFT correlations (transforms, vectors and partial
+ * sums FP32, totals and scalars FP64 or, at 512 pixels, 62-bit integers with an
+ * exponent). Updates d_spec in place; ORs APIC_TILE_NOTCONV into d_tile_status
+ * (may be NULL) where a solve ended above its tolerance. Tiles whose status has
+ * APIC_TILE_BACKGROUND or APIC_TILE_BADINPUT are left as they are.
  */
 apic_status apic_darkfield(apic_plan* plan, int n_tiles, const float* d_intensity,
                            const float* d_zernike, float* d_spec, int32_t* d_tile_status,
@@ -377,8 +380,10 @@ apic_status apic_simulate(apic_plan* plan, int n_tiles, const float* d_object,
  * the register-FFT and the shared-memory Stockham variants of the
  * Kramers-Kronig and darkfield stages (best of two runs after a warm-up, CUDA
  * events) and keeps the faster variant of each for the plan's later calls.
- * For 512-pixel tiles the register darkfield kernel is also timed with 1, 2
- * and 4 blocks (a thread-block cluster) per tile, and the fastest kept.
+ * For 512-pixel tiles the register darkfield kernel is also timed with 1 (and
+ * the rounds of apic_reconstruct_batch), 2 and 4 blocks (a thread-block
+ * cluster) per tile. A fixed 2 or 4 replaces the rounds for every later call,
+ * so it is kept only where it was faster on a sample of at least a full wave.
  * h_ms [n_ms] (may be NULL): milliseconds of KK register, KK Stockham,
  * darkfield register (the best cluster size), darkfield Stockham, and the
  * 512-pixel register darkfield kernel with 1, 2, 4 blocks per tile (-1 where

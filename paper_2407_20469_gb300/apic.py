@@ -347,7 +347,8 @@ class Plan:
 
     def autotune(self, n_tiles, intensity) -> dict:
         """Times the register and Stockham variants of the transform stages (and, for 512-pixel
-        tiles, the darkfield kernel with 1, 2, 4 blocks per tile) on a sample; keeps the fastest."""
+        tiles, the darkfield kernel with 1, 2, 4 blocks per tile) on a sample; keeps the fastest
+        (2 or 4 blocks only where the sample is at least a full wave)."""
         ms = np.full(7, -1.0)
         _check(load().apic_plan_autotune(self.handle, n_tiles, _ptr(intensity),
                                          ms.ctypes.data_as(C.POINTER(C.c_double)), 7), "apic_plan_autotune")

@@ -838,7 +838,8 @@ void split_geometry(const apic_plan* p, int nt, int& r, int& m0, int& ma, int& m
 // The darkfield stage runs one tile per block, so a chunk of nt tiles takes
 // ceil(nt / W) block rounds (W = blocks of a full wave) and its last partial
 // round leaves SMs idle. When nt is not a multiple of W, the r = nt mod W
-// trailing tiles go first: their earlier stages run, their darkfield solves
+// trailing tiles follow in rounds of clusters (launch_df) or, where hiding the
+// earlier stages gains more (df_rounds_beat_split), go first: their earlier stages run, their darkfield solves
 // start on a high-priority second stream (own scratch blocks), and meanwhile
 // the earlier stages of the other tiles run on the remaining SMs. Those tiles
 // then go to W - r blocks on the caller's stream (they start right away) and r

@@ -3,7 +3,7 @@
 //
 // The method, grids, transforms and the order of every sum are those of kernels_dfr.cu
 // (one block per tile), so a tile's result is bit for bit the same; this kernel is for
-// batches that leave SMs idle there. A tile is solved by K blocks (3 to 16): block r owns a
+// batches that leave SMs idle there. A tile is solved by K blocks (3 to 8): block r owns a
 // contiguous share of the grid's columns, of the Q rows and of the U rows.
 //  * No band grid of the CG leaves the cluster: a pass reads its rows or columns from the
 //    block's own shared memory and stores its results straight into the shared memory of

@@ -81,13 +81,13 @@ struct Layout {
 // keep the 64 columns kx in [-32, 32), forward transform of those columns,
 // keep ky in [-32, 32), log of the magnitude relative to the DC term (the
 // image sum). Output NHWC: feat[tile][ky + 32][kx + 32][image].
-// Three blocks of 256 threads per SM up to 256 pixels (as many as the scratch of n x n values
-// per SM holds), one of 512 at 512: at 256 pixels the kernel waits for its shared-memory
-// exchanges and loads, and 24 warps hide more of that than 16 do.
+// Blocks of 256 threads up to 256 pixels, as many per SM as the scratch of n x n values per SM
+// holds (three at 256 pixels, two at 128, one at 64), one of 512 at 512: at 256 pixels the kernel
+// waits for its shared-memory exchanges and loads, and 24 warps hide more of that than 16 do.
 // Bound by the L1 pipeline (the exchanges, twiddles and the kept columns' way through scratch).
 // The kept columns are stored in 4 x 4 tiles: a warp's load of two adjacent columns over 16
 // rows then touches 4 lines instead of 16. 512 tiles of 256 pixels 628 -> 484 us, of 128 354 -> 276,
-// 128 tiles of 512 pixels 507 -> 428.
+// 128 tiles of 512 pixels 507 -> 428 (2 % more since, for the image sum's rows in FP64).
 template <int BN>
 struct FeatCfg {
     static constexpr int threads = BN <= 16 ? 256 : 512, blocks = BN == 16 ? 3 : BN == 8 ? 2 : 1;
@@ -547,7 +547,8 @@ template <class L, class K, class... A>
 cudaError_t dgrad(K kernel, int B, long long* launches, cudaStream_t st, A... args) {
     return launch_layer<L>(kernel, dim3(B * L::tiles, L::gy), 256, launches, st, args...);
 }
-// about two blocks per SM over all channel tiles: each adds its sums to the gradient once
+// about one block per SM over all channel tiles (two in the first layer, whose blocks are small):
+// each adds its sums to the gradient once
 template <class L, class K, class... A>
 cudaError_t wgrad(K kernel, int B, long long* launches, cudaStream_t st, A... args) {
     const int img = L::C::IMG, tiles = (B + img - 1) / img * L::tiles;
