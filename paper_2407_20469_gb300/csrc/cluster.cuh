@@ -88,7 +88,9 @@ cudaError_t cluster_launch(void (*f)(P...), int K, int slots, int threads, size_
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
     cluster_config(cfg, attr, K, slots, threads, smem, st);
-    return cudaLaunchKernelEx(&cfg, f, args...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, f, args...);
+    if (e != cudaSuccess) cudaGetLastError();       // returned here, not by a later launch's check as well
+    return e;
 }
 
 }  // namespace apic
