@@ -695,7 +695,7 @@ def gpu_arm(args):
                    "launch": "direct C-ABI calls", "tiles_per_s": world * T * args.steps / (ms / 1e3),
                    "df_tol": args.df_tol or "library default", "fft_m": info.fft_m,
                    "precision": "FFTs, elementwise math and CG vectors FP32; aberration normal equations and "
-                                "darkfield CG step lengths / cross-warp sums FP64 (float pairs at 512 pixels)",
+                                "darkfield CG step lengths / cross-warp sums FP64 (62-bit integers with an exponent at 512 pixels)",
                    "tiles_status_nonzero": int(np.count_nonzero(status_np))},
         "roofline": roofline, "e2e": e2e, "gpu_launches": cnt["launches"], "clocks": clk,
     }
